@@ -204,6 +204,7 @@ struct cpic_run {
     bool graph_sort_fused[2][2];       // the graph's sort leaves its order to the next push
     cudaStream_t capture_stream;
     int cluster_cs;              // cluster size of the cluster solver (0: not applicable)
+    int cluster_nd;              // its split levels
     bool order_pending;          // a fused sort's order may be pending on the device (DevCounters::perm)
     bool count_hist;             // this step's direct 3D push and injection build the sort's histogram
     int dense_m;                 // coarsest unknowns (+1 row when singular)

@@ -86,6 +86,7 @@ struct LV {
     R* x;
     R* b;
     float* lw;  // 2D line relaxation: work [2][ncell] in global memory (FP32 levels)
+    const R* dinv;  // inverse diagonal (FP32 levels)
     const R* pw;  // 2D operator-induced prolongation: own-parent weight per axis [2][ncell], or null
 };
 
@@ -94,7 +95,7 @@ struct LVSet {
     int first_cta;  // first level solved inside one CTA
     int line;       // 1: alternating zebra line relaxation (2D) instead of point smoothing
     LV<float> l[MAX_LEVELS];
-    const float* dense_inv;
+    const float* dense_inv;  // transposed
     int dense_m;   // unknowns of the coarsest level
     int singular;
 };
@@ -263,7 +264,7 @@ __device__ __forceinline__ void restrict_at(const LV<R>& F, const LV<R>& Cl, con
 // and weights are set up once and combined per parent: w = ((1 w_0) w_1) w_2 and the signed
 // parent value, accumulated over the parents in order.
 template <int D, typename R>
-__device__ __forceinline__ void prolong_at(const LV<R>& F, const LV<R>& Cl, const int* q) {
+__device__ __forceinline__ R prolonged_at(const LV<R>& F, const LV<R>& Cl, const int* q) {
     const int f = q[0] + F.n[0] * (q[1] + F.n[1] * q[2]);
     R own[3] = {R(0.75), R(0.75), R(0.75)};  // weight of the own parent per axis (bilinear: 3/4)
     if (F.pw)
@@ -308,7 +309,11 @@ __device__ __forceinline__ void prolong_at(const LV<R>& F, const LV<R>& Cl, cons
         }
         acc += w * (sign * Cl.x[idx]);
     }
-    F.x[f] += acc;
+    return F.x[f] + acc;
+}
+template <int D, typename R>
+__device__ __forceinline__ void prolong_at(const LV<R>& F, const LV<R>& Cl, const int* q) {
+    F.x[q[0] + F.n[0] * (q[1] + F.n[1] * q[2])] = prolonged_at<D>(F, Cl, q);
 }
 
 // ------------------------------------------------------------------ line relaxation
@@ -619,41 +624,366 @@ __global__ void prolong_kernel(LV<float> F, LV<float> Cl) {
     prolong_at<D>(F, Cl, q);
 }
 
-// The lower part of the V-cycle (levels first_cta .. nl-1) inside one CTA, with every
-// level's stencil, inverse diagonal, correction and right-hand side in shared memory (the
-// top level's right-hand side comes from global memory, its correction goes back there).
-// All levels of a run share one stencil shape <D, NPT>.
-template <int D, int NPT>
-__global__ void __launch_bounds__(512) coarse_cycle_kernel(LVSet S, int nu1, int nu2) {
-    extern __shared__ float sm[];
-    __shared__ float sb[DENSE_MAX + 1];
-    __shared__ LV<float> V[MAX_LEVELS];
-    __shared__ float* Dv[MAX_LEVELS];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    if (tid == 0) {
-        int off = 0;
-        for (int l = S.first_cta; l < S.nl; ++l) {
-            V[l] = S.l[l];
-            V[l].A = sm + off;
-            off += NPT * S.l[l].ncell;
-            Dv[l] = sm + off;
-            off += S.l[l].ncell;
-            V[l].x = sm + off;
-            off += S.l[l].ncell;
-            V[l].b = sm + off;
-            off += S.l[l].ncell;
+// ---- one level's half of a V-cycle in one launch (2D, two colours)
+//
+// A block relaxes its tile of TL_X x TL_Y cells with TL_H cells of its surroundings: the four colour
+// sweeps of a V(2,2) half need no other block's values then, each leaving one ring of the
+// surroundings behind. So a level costs one launch on the way down (four sweeps from x = 0,
+// residual, restriction) and one on the way up (prolongation, four sweeps) in place of five
+// each, and its stencil is read once a launch and not once a sweep. A thread holds two pairs of
+// neighbouring cells (one cell of each colour) with their couplings in registers; x is in shared
+// memory with the colours of a row apart, so that a sweep's reads do not conflict. The tile: a
+// taller or wider one relaxes less twice (1.9 cells a cell here), a smaller one fills more of
+// the chip on the small levels, where the time is latency. On a 512 x 1024 V-cycle (levels
+// down to 64 x 128) a launch takes 3.9 us down and 4.7 us up on average, 82 us of sweeps,
+// transfers and memsets before.
+constexpr int TL_X = 32, TL_Y = 16, TL_H = 4, TL_THREADS = 256;
+constexpr int TL_W = TL_X + 2 * TL_H, TL_R = TL_Y + 2 * TL_H;  // cells of the extended tile
+constexpr int TL_HALF = TL_W / 2, TL_PAIRS = TL_HALF * TL_R;
+constexpr int TL_ITEMS = (TL_PAIRS + TL_THREADS - 1) / TL_THREADS;
+
+struct TilePair {
+    int at;            // shared offset of index m of the row's first colour (one row and word of margin)
+    int i, j;          // global cell of the pair's first cell (wrapped); i < 0: outside the domain
+    int ring;          // rings of the surroundings the pair lies in (0: own tile)
+    int odd;           // 1: its even cell is of the second colour
+    float a[2][4];     // couplings W, E, S, N per colour (the stencil's slots 1 .. 4)
+    float b[2], d[2];
+};
+
+// pair p of the extended tile of block (bx, by): its cells, couplings, right-hand side
+__device__ __forceinline__ void tile_pair(const LV<float>& L, int p, TilePair& t) {
+    const int r = p / TL_HALF, m = p - r * TL_HALF;
+    t.at = (r + 1) * TL_W + m + 1;
+    int i = (int)blockIdx.x * TL_X - TL_H + 2 * m, j = (int)blockIdx.y * TL_Y - TL_H + r;
+    const int x = 2 * m, rx = max(max(TL_H - x - 1, x - TL_H - TL_X + 1), 0), ry = max(max(TL_H - r, r - TL_H - TL_Y + 1), 0);
+    t.ring = max(rx, ry);  // of the pair's cell nearer to the tile
+    t.odd = j & 1;
+    bool in = p < TL_PAIRS;
+    if (L.per[0]) {
+        while (i < 0) i += L.n[0];
+        while (i >= L.n[0]) i -= L.n[0];
+    } else {
+        in = in && i >= 0 && i < L.n[0];
+    }
+    if (L.per[1]) {
+        while (j < 0) j += L.n[1];
+        while (j >= L.n[1]) j -= L.n[1];
+    } else {
+        in = in && j >= 0 && j < L.n[1];
+    }
+    t.i = in ? i : -1;
+    t.j = j;
+    const int c = in ? i + L.n[0] * j : 0, nc = L.ncell;
+    float2 z = make_float2(0.f, 0.f);
+    float2 w[4], bb, dd;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = in ? __ldg(reinterpret_cast<const float2*>(L.A + (k + 1) * nc + c)) : z;
+    bb = in ? *reinterpret_cast<const float2*>(L.b + c) : z;
+    dd = in ? __ldg(reinterpret_cast<const float2*>(L.dinv + c)) : z;
+    const bool o = t.odd != 0;  // colour 0 is the odd cell (2 m + 1) then
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        t.a[0][k] = o ? w[k].y : w[k].x;
+        t.a[1][k] = o ? w[k].x : w[k].y;
+    }
+    t.b[0] = o ? bb.y : bb.x;
+    t.b[1] = o ? bb.x : bb.y;
+    t.d[0] = o ? dd.y : dd.x;
+    t.d[1] = o ? dd.x : dd.y;
+}
+
+// s + couplings times neighbours of the pair's cell of colour C, in the order of stencil_sum
+template <int C>
+__device__ __forceinline__ float tile_sum(const TilePair& t, const float* x, float s) {
+    const float* o = x + t.at + (1 - C) * TL_HALF;
+    const bool even = (C == 0) != (t.odd != 0);  // the cell is 2 m: its pair neighbour is to the east
+    s += t.a[C][0] * o[even ? -1 : 0];
+    s += t.a[C][1] * o[even ? 0 : 1];
+    s += t.a[C][2] * o[-TL_W];
+    s += t.a[C][3] * o[TL_W];
+    return s;
+}
+template <int C>
+__device__ __forceinline__ float tile_relaxed(const TilePair& t, const float* x) {
+    return (t.b[C] - tile_sum<C>(t, x, 0.0f)) * t.d[C];
+}
+
+// the ring of the pair's cell of colour C (a pair astride a column of rings: its outer cell is one
+// further out)
+template <int C>
+__device__ __forceinline__ int ring_of(const TilePair& t, int p) {
+    const int r = p / TL_HALF, m = p - r * TL_HALF;
+    const int x = 2 * m + (((C == 0) != (t.odd != 0)) ? 0 : 1);
+    return max(max(TL_H - x, x - TL_H - TL_X + 1), max(max(TL_H - r, r - TL_H - TL_Y + 1), 0));
+}
+
+// Down: x = 0, sweeps of colours 0, 1, 0, 1, then Cl.b = sums of the residuals, in the order of
+// restrict_at. x keeps the first colour only: the way up prolongs onto it and relaxes the
+// second from it.
+__global__ void __launch_bounds__(TL_THREADS) level_down2_kernel(const __grid_constant__ LV<float> L, float* bc, int cn0) {
+    __shared__ float x[(TL_R + 2) * TL_W + 2];
+    __shared__ float rs[TL_Y][TL_X];
+    const int tid = threadIdx.x;
+    for (int e = tid; e < (TL_R + 2) * TL_W + 2; e += TL_THREADS) x[e] = 0.0f;
+    TilePair t[TL_ITEMS];
+#pragma unroll
+    for (int u = 0; u < TL_ITEMS; ++u) tile_pair(L, tid + u * TL_THREADS, t[u]);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int u = 0; u < TL_ITEMS; ++u) {
+            const int p = tid + u * TL_THREADS;
+            if (p >= TL_PAIRS) continue;
+            if (k & 1) {
+                if (ring_of<1>(t[u], p) <= TL_H - k) x[t[u].at + TL_HALF] = tile_relaxed<1>(t[u], x);
+            } else if (ring_of<0>(t[u], p) <= TL_H - k) {
+                x[t[u].at] = k ? tile_relaxed<0>(t[u], x) : t[u].b[0] * t[u].d[0];
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < TL_ITEMS; ++u) {
+        const int p = tid + u * TL_THREADS;
+        if (p >= TL_PAIRS || t[u].ring) continue;
+        const int r = p / TL_HALF - TL_H, m = p % TL_HALF - TL_H / 2;
+        const int gi = (int)blockIdx.x * TL_X + 2 * m, gj = (int)blockIdx.y * TL_Y + r;
+        if (gi >= L.n[0] || gj >= L.n[1]) continue;
+        const float2 dg = __ldg(reinterpret_cast<const float2*>(L.A + gi + L.n[0] * gj));
+        const float x0 = x[t[u].at], x1 = x[t[u].at + TL_HALF];
+        const int o = t[u].odd;
+        rs[r][2 * m + o] = t[u].b[0] - tile_sum<0>(t[u], x, __fmul_rn(o ? dg.y : dg.x, x0));
+        rs[r][2 * m + 1 - o] = t[u].b[1] - tile_sum<1>(t[u], x, __fmul_rn(o ? dg.x : dg.y, x1));
+        L.x[gi + o + L.n[0] * gj] = x0;
+    }
+    __syncthreads();
+    if (tid < TL_X / 2 * (TL_Y / 2)) {
+        const int ic = tid % (TL_X / 2), jc = tid / (TL_X / 2);
+        const int I = (int)blockIdx.x * (TL_X / 2) + ic, J = (int)blockIdx.y * (TL_Y / 2) + jc;
+        if (2 * I < L.n[0] && 2 * J < L.n[1])
+            bc[I + cn0 * J] = ((rs[2 * jc][2 * ic] + rs[2 * jc][2 * ic + 1]) + rs[2 * jc + 1][2 * ic]) + rs[2 * jc + 1][2 * ic + 1];
+    }
+}
+
+// Up: prolongation onto the first colour, sweeps of colours 1, 0, 1, 0, result into xo (other
+// blocks read this level's x meanwhile)
+__global__ void __launch_bounds__(TL_THREADS) level_up2_kernel(const __grid_constant__ LV<float> L, const __grid_constant__ LV<float> Cl,
+                                                               float* xo) {
+    __shared__ float x[(TL_R + 2) * TL_W + 2];
+    const int tid = threadIdx.x;
+    for (int e = tid; e < (TL_R + 2) * TL_W + 2; e += TL_THREADS) x[e] = 0.0f;
+    TilePair t[TL_ITEMS];
+    float v[TL_ITEMS];
+#pragma unroll
+    for (int u = 0; u < TL_ITEMS; ++u) {
+        tile_pair(L, tid + u * TL_THREADS, t[u]);
+        v[u] = 0.0f;
+        if (t[u].i >= 0) {
+            const int q[3] = {t[u].i + t[u].odd, t[u].j, 0};
+            v[u] = prolonged_at<2>(L, Cl, q);
         }
     }
     __syncthreads();
-    for (int l = S.first_cta; l < S.nl; ++l) {
-        const LV<float>& G = S.l[l];
-        float* A = const_cast<float*>(V[l].A);
-        for (int e = tid; e < NPT * G.ncell; e += nt) A[e] = G.A[e];
-        for (int c = tid; c < G.ncell; c += nt) {
-            Dv[l][c] = 1.0f / G.A[c];
-            V[l].x[c] = 0.0f;
-            if (l == S.first_cta) V[l].b[c] = G.b[c];
+#pragma unroll
+    for (int u = 0; u < TL_ITEMS; ++u)
+        if (tid + u * TL_THREADS < TL_PAIRS) x[t[u].at] = v[u];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int u = 0; u < TL_ITEMS; ++u) {
+            const int p = tid + u * TL_THREADS;
+            if (p >= TL_PAIRS) continue;
+            if (k & 1) {
+                if (ring_of<0>(t[u], p) < TL_H - k) x[t[u].at] = tile_relaxed<0>(t[u], x);
+            } else if (ring_of<1>(t[u], p) < TL_H - k) {
+                x[t[u].at + TL_HALF] = tile_relaxed<1>(t[u], x);
+            }
         }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < TL_ITEMS; ++u) {
+        const int p = tid + u * TL_THREADS;
+        if (p >= TL_PAIRS || t[u].ring) continue;
+        const int r = p / TL_HALF - TL_H, m = p % TL_HALF - TL_H / 2;
+        const int gi = (int)blockIdx.x * TL_X + 2 * m, gj = (int)blockIdx.y * TL_Y + r;
+        if (gi >= L.n[0] || gj >= L.n[1]) continue;
+        const float c0 = x[t[u].at], c1 = x[t[u].at + TL_HALF];
+        *reinterpret_cast<float2*>(xo + gi + L.n[0] * gj) = t[u].odd ? make_float2(c1, c0) : make_float2(c0, c1);
+    }
+}
+
+// ---- the lower part of the V-cycle (levels first_cta .. nl-1) inside one CTA
+
+// sizes of a level in the one-CTA part, with multipliers for its index divisions
+struct CtaLevel {
+    int n0, n1, n2, half, ncell;
+    unsigned mh, m1;  // idx / half, idx / n1 as __umulhi (0: the divisor is 1)
+    float *A, *dinv, *x, *b;
+};
+
+__device__ __forceinline__ unsigned div_magic(int d) { return d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u; }
+__device__ __forceinline__ int div_by(int idx, unsigned magic) { return magic ? (int)__umulhi((unsigned)idx, magic) : idx; }
+
+// steps from a cell to its neighbours along each axis. They wrap on every axis: where an axis
+// is not periodic the stencil entry of a neighbour beyond the face is zero.
+template <int D>
+struct Steps {
+    int lo[3], hi[3];
+    __device__ __forceinline__ Steps(const CtaLevel& L, int i, int j, int k) {
+        lo[0] = i > 0 ? -1 : L.n0 - 1;
+        hi[0] = i < L.n0 - 1 ? 1 : 1 - L.n0;
+        lo[1] = (j > 0 ? -1 : L.n1 - 1) * L.n0;
+        hi[1] = (j < L.n1 - 1 ? 1 : 1 - L.n1) * L.n0;
+        if (D == 3) {
+            const int pl = L.n0 * L.n1;
+            lo[2] = (k > 0 ? -1 : L.n2 - 1) * pl;
+            hi[2] = (k < L.n2 - 1 ? 1 : 1 - L.n2) * pl;
+        }
+    }
+    __device__ __forceinline__ int operator()(int slot) const {  // constant arguments: folds away
+        int o = 0;
+#pragma unroll
+        for (int a = 0; a < D; ++a) o += koff(D, slot, a) < 0 ? lo[a] : (koff(D, slot, a) > 0 ? hi[a] : 0);
+        return o;
+    }
+};
+
+// sum of the stencil's entries from K0 on times their cells, in the order of stencil_sum (the
+// Krylov iteration amplifies a rounding to the size of its stopping error, so every form of
+// the V-cycle keeps to one order of operations)
+template <int D, int NPT, int K0>
+__device__ __forceinline__ float cta_sum(const CtaLevel& L, int c, const Steps<D>& st) {
+    float acc = 0.0f;
+#pragma unroll
+    for (int k = K0; k < NPT; ++k) acc += L.A[k * L.ncell + c] * L.x[c + st(k)];
+    return acc;
+}
+
+// One colour of a level. The cells of a colour are (m, j, k) with a half-length first axis (and
+// half-length other axes when the stencil has 2^D colours); first: x = 0 everywhere else.
+template <int D, int NPT>
+__device__ __forceinline__ void cta_sweep(const CtaLevel& L, int colour, bool first) {
+    constexpr bool parity = Col<D, NPT>::parity;
+    const int d1 = parity ? L.n1 : L.n1 / 2, d2 = D == 3 ? (parity ? L.n2 : L.n2 / 2) : 1;
+    const unsigned m1 = parity ? L.m1 : div_magic(d1);
+    const int count = L.half * d1 * d2;
+    for (int idx = threadIdx.x; idx < count; idx += blockDim.x) {
+        const int row = div_by(idx, L.mh), m = idx - row * L.half;
+        const int k = D == 3 ? div_by(row, m1) : 0, j = row - k * d1;
+        int q[3];
+        Col<D, NPT>::cell(colour, m, j, k, q);
+        const int c = q[0] + L.n0 * (q[1] + L.n1 * q[2]);
+        const float s = first ? 0.0f : cta_sum<D, NPT, 1>(L, c, Steps<D>(L, q[0], q[1], q[2]));
+        L.x[c] = (L.b[c] - s) * L.dinv[c];
+    }
+    __syncthreads();
+}
+
+// Cl.b = sum of the children's residuals, in the order of restrict_at
+template <int D, int NPT>
+__device__ __forceinline__ void cta_restrict(const CtaLevel& F, const CtaLevel& Cl) {
+    for (int C = threadIdx.x; C < Cl.ncell; C += blockDim.x) {
+        const int row = div_by(C, F.mh), ic = C - row * Cl.n0;  // Cl.n0 = F.half
+        const int kc = D == 3 ? row / Cl.n1 : 0, jc = row - kc * Cl.n1;
+        float acc = 0.0f;
+#pragma unroll
+        for (int ch = 0; ch < (D == 2 ? 4 : 8); ++ch) {
+            const int i = 2 * ic + (ch & 1), j = 2 * jc + ((ch >> 1) & 1), k = D == 3 ? 2 * kc + ((ch >> 2) & 1) : 0;
+            const int c = i + F.n0 * (j + F.n1 * k);
+            acc += F.b[c] - cta_sum<D, NPT, 0>(F, c, Steps<D>(F, i, j, k));
+        }
+        Cl.b[C] = acc;
+        Cl.x[C] = 0.0f;
+    }
+    __syncthreads();
+}
+
+// All of these levels' stencils, inverse diagonals and right-hand sides come in by bulk copies
+// (one a level and array, so the load is one latency and not a chain of them); with the dense
+// inverse beside them when it fits; the first sweep from x = 0 reads no neighbours, and of two
+// colours the second is not prolonged onto (the next sweep overwrites it). The CTA part of a
+// 512 x 1024 V-cycle (levels of 32 x 64 cells and below) takes 16 us (33 with per-cell
+// index divisions, element-wise staging and the dense inverse read a row per thread), that of
+// a 24 x 20 x 16 one (12 x 10 x 8 and below) 10.5 us (18.8).
+template <int D, int NPT>
+__global__ void __launch_bounds__(512, 1) coarse_cycle_kernel(const __grid_constant__ LVSet S, int nu1, int nu2, int dense_smem) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ LV<float> V[MAX_LEVELS];
+    __shared__ CtaLevel T[MAX_LEVELS];
+    __shared__ __align__(8) unsigned long long bar;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int m = S.dense_m, mm = m + (S.singular ? 1 : 0);
+    const unsigned ubar = (unsigned)__cvta_generic_to_shared(&bar);
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(ubar) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        // shared memory: per level A [NPT], dinv, x, b (a multiple of four words each on the
+        // smoothed levels, whose axes are even); then the dense inverse
+        int off = 0;
+        unsigned bytes = 0;
+        for (int l = S.first_cta; l < S.nl; ++l) {
+            const LV<float>& G = S.l[l];
+            const int nc = (G.ncell + 3) & ~3;
+            V[l] = G;
+            CtaLevel& L = T[l];
+            L.n0 = G.n[0], L.n1 = G.n[1], L.n2 = G.n[2], L.half = G.n[0] / 2, L.ncell = G.ncell;
+            L.mh = div_magic(L.half);
+            L.m1 = div_magic(L.n1);
+            if (l < S.nl - 1) {
+                L.A = sm + off;
+                L.dinv = L.A + NPT * nc;
+                L.x = L.dinv + nc;
+                off += (NPT + 2) * nc;
+                bytes += (NPT + 1) * G.ncell * 4;
+            } else {  // the dense level needs its right-hand side and solution only
+                L.A = L.dinv = nullptr;
+                L.x = sm + off;
+                off += nc;
+            }
+            L.b = sm + off;
+            off += nc;
+            V[l].A = L.A;
+            V[l].x = L.x;
+            V[l].b = L.b;
+        }
+        const bool smoothed = S.first_cta < S.nl - 1;
+        if (smoothed) bytes += S.l[S.first_cta].ncell * 4;  // its right-hand side
+        const unsigned dense_bytes = dense_smem ? (unsigned)((mm * mm * 4 + 15) & ~15) : 0u;
+        bytes += dense_bytes;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(ubar), "r"(bytes) : "memory");
+        auto copy = [&](float* dst, const float* src, unsigned n) {
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(dst)),
+                         "l"(src), "r"(n), "r"(ubar)
+                         : "memory");
+        };
+        for (int l = S.first_cta; l < S.nl - 1; ++l) {
+            const int nc = S.l[l].ncell;
+            copy(T[l].A, S.l[l].A, NPT * nc * 4);
+            copy(T[l].dinv, S.l[l].dinv, nc * 4);
+        }
+        if (smoothed) copy(T[S.first_cta].b, S.l[S.first_cta].b, S.l[S.first_cta].ncell * 4);
+        if (dense_smem) copy(sm + dense_smem, S.dense_inv, dense_bytes);
+    }
+    __syncthreads();
+    for (int c = tid; c < T[S.first_cta].ncell; c += nt) {
+        T[S.first_cta].x[c] = 0.0f;
+        if (S.first_cta == S.nl - 1) T[S.first_cta].b[c] = S.l[S.first_cta].b[c];
+    }
+    {
+        // the copies take a microsecond or so: a bounded wait (on giving up the values are wrong,
+        // the residual does not fall and the solve reports it)
+        unsigned done = 0;
+        for (int spin = 0; spin < (1 << 20) && !done; ++spin)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done)
+                : "r"(ubar)
+                : "memory");
     }
     __syncthreads();
     // alternating zebra line relaxation: lines along each axis in turn, each colour in turn
@@ -675,68 +1005,66 @@ __global__ void __launch_bounds__(512) coarse_cycle_kernel(LVSet S, int nu1, int
             }
         }
     };
-    auto sweep = [&](int l, int col) {
-        const LV<float>& L = V[l];
-        int d[3];
-        Col<D, NPT>::dims(L, d);
-        const int plane = d[0] * d[1];
-        for (int idx = tid; idx < plane * d[2]; idx += nt) {
-            int k = idx / plane, r = idx - k * plane;
-            int j = r / d[0], m = r - j * d[0];
-            int q[3];
-            Col<D, NPT>::cell(col, m, j, k, q);
-            smooth_at<D, NPT>(L, (const float*)Dv[l], q);
-        }
-        __syncthreads();
-    };
+    constexpr int NCOL = Col<D, NPT>::parity ? 2 : 1 << D;
     for (int l = S.first_cta; l < S.nl - 1; ++l) {
+        const CtaLevel L = T[l];
         for (int it = 0; it < nu1; ++it) {
             if (S.line) line_sweep(l, false);
             else
-                for (int col = 0; col < V[l].ncol; ++col) sweep(l, col);
+                for (int col = 0; col < NCOL; ++col) cta_sweep<D, NPT>(L, col, it == 0 && col == 0);
         }
-        const LV<float>& C = V[l + 1];
-        const int plane = C.n[0] * C.n[1];
-        for (int idx = tid; idx < C.ncell; idx += nt) {
-            int k = idx / plane, r = idx - k * plane;
-            int j = r / C.n[0];
-            int q[3] = {r - j * C.n[0], j, k};
-            restrict_at<D, NPT>(V[l], C, q);
+        if (S.line) {
+            // every cell has a residual after a line sweep
+            const LV<float>& C = V[l + 1];
+            const int plane = C.n[0] * C.n[1];
+            for (int idx = tid; idx < C.ncell; idx += nt) {
+                const int k = idx / plane, r = idx - k * plane, j = r / C.n[0];
+                const int q[3] = {r - j * C.n[0], j, k};
+                restrict_at<D, NPT>(V[l], C, q);
+            }
+            __syncthreads();
+        } else {
+            cta_restrict<D, NPT>(L, T[l + 1]);
         }
-        __syncthreads();
     }
     {
-        const LV<float>& L = V[S.nl - 1];
-        int m = S.dense_m;
-        int mm = m + (S.singular ? 1 : 0);
-        for (int i = tid; i < mm; i += nt) sb[i] = i < m ? L.b[i] : 0.0f;
-        __syncthreads();
+        // dense solve, one unknown a thread (the inverse is stored transposed, so that
+        // neighbouring threads read neighbours)
+        const float* bs = T[S.nl - 1].b;
         for (int i = tid; i < m; i += nt) {
-            const float* row = S.dense_inv + i * mm;
             float acc = 0.0f;
-            for (int k = 0; k < mm; ++k) acc += row[k] * sb[k];
-            L.x[i] = acc;
+            if (dense_smem) {
+                const float* R = sm + dense_smem + i;
+#pragma unroll 8
+                for (int k = 0; k < m; ++k) acc += R[k * mm] * bs[k];
+            } else {
+#pragma unroll 16
+                for (int k = 0; k < m; ++k) acc += __ldg(S.dense_inv + k * mm + i) * bs[k];
+            }
+            T[S.nl - 1].x[i] = acc;
         }
         __syncthreads();
     }
     for (int l = S.nl - 2; l >= S.first_cta; --l) {
         const LV<float>& L = V[l];
-        const int plane = L.n[0] * L.n[1];
-        for (int idx = tid; idx < L.ncell; idx += nt) {
-            int k = idx / plane, r = idx - k * plane;
-            int j = r / L.n[0];
-            int q[3] = {r - j * L.n[0], j, k};
+        const CtaLevel F = T[l];
+        for (int idx = tid; idx < F.ncell; idx += nt) {
+            const int row = div_by(idx >> 1, F.mh), i = idx - row * F.n0;
+            const int k = D == 3 ? div_by(row, F.m1) : 0, j = row - k * F.n1;
+            // with two colours the next sweep overwrites the second
+            if (!S.line && Col<D, NPT>::parity && ((i + j + k) & 1)) continue;
+            const int q[3] = {i, j, k};
             prolong_at<D>(L, V[l + 1], q);
         }
         __syncthreads();
         for (int it = 0; it < nu2; ++it) {
             if (S.line) line_sweep(l, true);
             else
-                for (int col = V[l].ncol - 1; col >= 0; --col) sweep(l, col);
+                for (int col = NCOL - 1; col >= 0; --col) cta_sweep<D, NPT>(F, col, false);
         }
     }
-    const LV<float>& T = S.l[S.first_cta];
-    for (int c = tid; c < T.ncell; c += nt) T.x[c] = V[S.first_cta].x[c];
+    const LV<float>& G = S.l[S.first_cta];
+    for (int c = tid; c < G.ncell; c += nt) G.x[c] = T[S.first_cta].x[c];
 }
 
 // ------------------------------------------------------------------ FP64 outer iteration
@@ -1213,6 +1541,14 @@ __global__ void to_float_kernel(const double* src, float* dst, long long n) {
         dst[i] = (float)src[i];
 }
 
+// dst = src^T, rounded to FP32 (the dense inverse, as the coarse solves read it)
+__global__ void to_float_transposed_kernel(const double* src, float* dst, int n) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * n; e += gridDim.x * blockDim.x) {
+        const int i = e / n, k = e - i * n;
+        dst[k * n + i] = (float)src[e];
+    }
+}
+
 // dense matrix of the coarsest level (bordered with ones when singular), row-major mm x mm
 __global__ void dense_matrix_kernel(LV<double> L, int singular, double* M) {
     int m = (int)L.ncell, mm = m + (singular ? 1 : 0);
@@ -1315,7 +1651,9 @@ LV<R> make_lv(const cpic_run* r, int l, bool fp32) {
         L.A = (const R*)Lv.A32;
         L.x = (R*)Lv.x32;
         L.b = (R*)Lv.b32;
+        L.dinv = (const R*)Lv.dinv32;
     } else {
+        L.dinv = nullptr;
         L.A = (const R*)Lv.A;
         L.x = (R*)Lv.x;
         L.b = (R*)Lv.b;
@@ -1332,30 +1670,43 @@ int grid_blocks(long long n, int threads) {
 
 constexpr size_t CTA_SMEM_MAX = 200 * 1024;  // shared memory of the one-CTA coarse cycle
 
+// words of the one-CTA part from level l on: stencil (of the finest level's shape on every
+// level), inverse diagonal, x, b of every smoothed level, x and b of the dense one
+size_t cta_words(const LVSet& S, int l) {
+    size_t f = 0;
+    for (int k = l; k < S.nl; ++k) f += (size_t)(k < S.nl - 1 ? S.l[0].used + 3 : 2) * ((S.l[k].ncell + 3) & ~3);
+    return f;
+}
+
 LVSet make_set(const cpic_run* r) {
     LVSet S;
     S.nl = r->nlevels;
     S.line = r->mg_smoother == CPIC_MG_SMOOTH_LINE ? 1 : 0;
     for (int l = 0; l < r->nlevels; ++l) S.l[l] = make_lv<float>(r, l, true);
-    // the one-CTA part starts at the first level of at most COARSE_CELLS cells from which
-    // every coarser level fits the CTA's shared memory (stencil, inverse diagonal, x, b)
-    S.first_cta = r->nlevels - 1;
-    for (int l = r->nlevels - 1; l >= 0; --l) {
-        if (r->lev[l].ncell > COARSE_CELLS) break;
-        size_t f = 0;
-        for (int k = l; k < r->nlevels; ++k) f += (size_t)(S.l[k].used + 3) * S.l[k].ncell;
-        if (f * sizeof(float) > CTA_SMEM_MAX) break;
-        S.first_cta = l;
-    }
     S.dense_inv = r->dense_inv32;
     S.dense_m = (int)r->lev[r->nlevels - 1].ncell;
     S.singular = r->singular ? 1 : 0;
+    // the one-CTA part starts at the first level of at most COARSE_CELLS cells from which
+    // every coarser level fits the CTA's shared memory
+    S.first_cta = r->nlevels - 1;
+    for (int l = r->nlevels - 1; l >= 0; --l) {
+        if (r->lev[l].ncell > COARSE_CELLS) break;
+        if (cta_words(S, l) * sizeof(float) > CTA_SMEM_MAX) break;
+        S.first_cta = l;
+    }
     return S;
 }
 
-size_t cta_smem_bytes(const LVSet& S) {
-    size_t f = 0;
-    for (int l = S.first_cta; l < S.nl; ++l) f += (size_t)(S.l[l].used + 3) * S.l[l].ncell;
+// shared memory of the one-CTA part; dense: the offset (words) of the dense inverse in it, 0 when it
+// does not fit
+size_t cta_smem_bytes(const LVSet& S, int* dense) {
+    size_t f = cta_words(S, S.first_cta);
+    const size_t mm = S.dense_m + S.singular, with = f + ((mm * mm + 3) & ~size_t(3));
+    *dense = 0;
+    if (with * sizeof(float) <= CTA_SMEM_MAX) {
+        *dense = (int)f;
+        f = with;
+    }
     return f * sizeof(float);
 }
 
@@ -1400,14 +1751,56 @@ int dispatch_vshape(const cpic_run* r, F f) {
                  : f(std::integral_constant<int, 3>(), std::integral_constant<int, 7>());
 }
 
-// one FP32 V-cycle on the correction equation (e = 0 first): lev[0].x32 = V(lev[0].b32)
+// the levels of the one-CTA part
+template <int D, int NPT>
+int enqueue_coarse(cpic_run* r, const LVSet& S, int nu1, int nu2) {
+    int dense = 0;
+    const size_t smem = cta_smem_bytes(S, &dense);
+    if (smem > CTA_SMEM_MAX) {
+        set_error("multigrid: coarse levels need %zu bytes of shared memory", smem);
+        return CPIC_ERR_INVALID;
+    }
+    // per-function attribute shared by every run (and by graphs captured earlier): set it
+    // to the bound checked above, not to this run's need
+    CPIC_CUDA(cudaFuncSetAttribute(coarse_cycle_kernel<D, NPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)CTA_SMEM_MAX));
+    coarse_cycle_kernel<D, NPT><<<1, 512, smem, r->stream>>>(S, nu1, nu2, dense);
+    CPIC_CHECK_LAUNCH();
+    return CPIC_OK;
+}
+
+// whether the V-cycle takes one launch per level and direction (2D, two colours, point smoothing)
+bool fused_levels(const LVSet& S) { return S.l[0].D == 2 && S.l[0].used == 5 && !S.line; }
+// where the V-cycle leaves level l's correction
+float* vcycle_result(const LVSet& S, int l) { return fused_levels(S) && l < S.first_cta ? S.l[l].lw : S.l[l].x; }
+
+// one FP32 V-cycle on the correction equation (e = 0 first): vcycle_result(S, 0) = V(lev[0].b32)
 int enqueue_vcycle(cpic_run* r, const LVSet& S) {
     return dispatch_vshape(r, [&](auto Dc, auto Nc) -> int {
         constexpr int D = decltype(Dc)::value, NPT = decltype(Nc)::value;
         cudaStream_t st = r->stream;
         const int nu1 = 2, nu2 = 2;
-        CPIC_CUDA(cudaMemsetAsync(r->lev[0].x32, 0, sizeof(float) * r->lev[0].ncell, st));
         const int top = S.first_cta;
+        // 2D two-colour levels: one launch down and one up each, the results in the levels' second
+        // buffers (the line-relaxation work, free with point smoothing)
+        if (D == 2 && NPT == 5 && fused_levels(S)) {
+            auto tiles = [&](int l) {
+                return dim3((unsigned)((S.l[l].n[0] + TL_X - 1) / TL_X), (unsigned)((S.l[l].n[1] + TL_Y - 1) / TL_Y));
+            };
+            for (int l = 0; l < top; ++l) {
+                level_down2_kernel<<<tiles(l), TL_THREADS, 0, st>>>(S.l[l], S.l[l + 1].b, S.l[l + 1].n[0]);
+                CPIC_CHECK_LAUNCH();
+            }
+            if (int e = enqueue_coarse<D, NPT>(r, S, nu1, nu2)) return e;
+            for (int l = top - 1; l >= 0; --l) {
+                LV<float> C = S.l[l + 1];
+                C.x = vcycle_result(S, l + 1);
+                level_up2_kernel<<<tiles(l), TL_THREADS, 0, st>>>(S.l[l], C, vcycle_result(S, l));
+                CPIC_CHECK_LAUNCH();
+            }
+            return CPIC_OK;
+        }
+        CPIC_CUDA(cudaMemsetAsync(r->lev[0].x32, 0, sizeof(float) * r->lev[0].ncell, st));
         auto smooth = [&](int l, int col) -> int {
             const LV<float>& L = S.l[l];
             int d[3] = {L.n[0] / 2, Col<D, NPT>::parity ? L.n[1] : L.n[1] / 2,
@@ -1450,17 +1843,7 @@ int enqueue_vcycle(cpic_run* r, const LVSet& S) {
             restrict_kernel<D, NPT><<<rg, rb, 0, st>>>(Fl, C);
             CPIC_CHECK_LAUNCH();
         }
-        size_t smem = cta_smem_bytes(S);
-        if (smem > CTA_SMEM_MAX) {
-            set_error("multigrid: coarse levels need %zu bytes of shared memory", smem);
-            return CPIC_ERR_INVALID;
-        }
-        // per-function attribute shared by every run (and by graphs captured earlier): set it
-        // to the bound checked above, not to this run's need
-        CPIC_CUDA(cudaFuncSetAttribute(coarse_cycle_kernel<D, NPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)CTA_SMEM_MAX));
-        coarse_cycle_kernel<D, NPT><<<1, 512, smem, st>>>(S, nu1, nu2);
-        CPIC_CHECK_LAUNCH();
+        if (int e = enqueue_coarse<D, NPT>(r, S, nu1, nu2)) return e;
         for (int l = top - 1; l >= 0; --l) {
             const LV<float>& L = S.l[l];
             prolong_kernel<D><<<cell_grid(L.n[0], L.n[1], L.n[2]), kCellBlock, 0, st>>>(L, S.l[l + 1]);
@@ -1482,7 +1865,7 @@ int enqueue_vcycle(cpic_run* r, const LVSet& S) {
 int enqueue_correction(cpic_run* r, const LVSet& S) {
     int st = enqueue_vcycle(r, S);
     if (st) return st;
-    update_kernel<<<grid_blocks(r->lev[0].ncell, 256), 256, 0, r->stream>>>(r->lev[0].x, r->lev[0].x32,
+    update_kernel<<<grid_blocks(r->lev[0].ncell, 256), 256, 0, r->stream>>>(r->lev[0].x, vcycle_result(S, 0),
                                                                             (int)r->lev[0].ncell);
     CPIC_CHECK_LAUNCH();
     return CPIC_OK;
@@ -1525,7 +1908,7 @@ int enqueue_bicg_iteration(cpic_run* r, const LVSet& S, double rtol, int max_cyc
     float* v = p + r->ncell;
     float* s = v + r->ncell;
     float* b32 = r->lev[0].b32;
-    float* x32 = r->lev[0].x32;
+    const float* x32 = vcycle_result(S, 0);
     cudaStream_t st = r->stream;
     const int gb = grid_blocks(n, 256);
     bicg_direction_kernel<<<gb, 256, 0, st>>>(n, rv, rh, p, v, b32, r->kry);
@@ -1668,8 +2051,7 @@ int mg_setup(cpic_run* r) {
     CPIC_CUDA(cudaMemsetAsync(fail, 0, sizeof(int), r->stream));
     gauss_jordan_kernel<<<1, 1024, 0, r->stream>>>(r->dense_tmp, r->dense_inv, mm, fail);
     CPIC_CHECK_LAUNCH();
-    to_float_kernel<<<grid_blocks((long long)mm * mm, 256), 256, 0, r->stream>>>(r->dense_inv, r->dense_inv32,
-                                                                                  (long long)mm * mm);
+    to_float_transposed_kernel<<<grid_blocks((long long)mm * mm, 256), 256, 0, r->stream>>>(r->dense_inv, r->dense_inv32, mm);
     CPIC_CHECK_LAUNCH();
     CPIC_CUDA(cudaMemsetAsync(r->ticket, 0, sizeof(unsigned) * 4, r->stream));
     CPIC_CUDA(cudaMemsetAsync(r->kry, 0, sizeof(KrylovState), r->stream));

@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) mg_cluster_kernel(const __grid_
                 else __syncthreads();
             }
             {
-                // dense solve; the inverse is symmetric, so the threads read it along its rows
+                // dense solve (the inverse is stored transposed)
                 const int ob = P.L[P.nl - 1].ob, ox = P.L[P.nl - 1].ox;
                 float* ps = sm + P.odense;
                 if (dense_regs) {

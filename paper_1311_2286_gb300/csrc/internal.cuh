@@ -205,6 +205,7 @@ struct cpic_run {
     cudaStream_t capture_stream;
     int cluster_cs;              // cluster size of the cluster solver (0: not applicable)
     int cluster_nd;              // its split levels
+    int slab_cs;                 // largest cluster of the 3D V-cycle's cluster part (0: none)
     bool order_pending;          // a fused sort's order may be pending on the device (DevCounters::perm)
     bool count_hist;             // this step's direct 3D push and injection build the sort's histogram
     int dense_m;                 // coarsest unknowns (+1 row when singular)

@@ -45,6 +45,7 @@
 // it writes the decision into a CUDA graph conditional handle, so inside a captured step
 // the cycle loop is a conditional WHILE node that runs on the device with no host round
 // trip and no idle launches.
+#include <cooperative_groups.h>
 #include <stdlib.h>
 #include <math.h>
 #include <string.h>
@@ -52,6 +53,8 @@
 #include <type_traits>
 
 #include "internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace cpic {
 namespace {
@@ -902,90 +905,80 @@ __device__ __forceinline__ void cta_restrict(const CtaLevel& F, const CtaLevel& 
     __syncthreads();
 }
 
-// All of these levels' stencils, inverse diagonals and right-hand sides come in by bulk copies
-// (one a level and array, so the load is one latency and not a chain of them); with the dense
-// inverse beside them when it fits; the first sweep from x = 0 reads no neighbours, and of two
-// colours the second is not prolonged onto (the next sweep overwrites it). The CTA part of a
-// 512 x 1024 V-cycle (levels of 32 x 64 cells and below) takes 16 us (33 with per-cell
-// index divisions, element-wise staging and the dense inverse read a row per thread), that of
-// a 24 x 20 x 16 one (12 x 10 x 8 and below) 10.5 us (18.8).
+// mbarrier with one arrival, and bulk copies from global memory that complete on it
+struct BulkLoad {
+    unsigned bar;
+    unsigned bytes;
+    __device__ __forceinline__ void init(unsigned long long* b) {
+        bar = (unsigned)__cvta_generic_to_shared(b);
+        bytes = 0;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __device__ __forceinline__ void copy(float* dst, const float* src, unsigned n) {
+        bytes += n;
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(dst)),
+                     "l"(src), "r"(n), "r"(bar)
+                     : "memory");
+    }
+    __device__ __forceinline__ void arrive() const {
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    }
+};
+// every thread waits for the copies: a microsecond or so, with a limit (on giving up the values are
+// wrong, the residual does not fall and the solve reports it)
+__device__ __forceinline__ void bulk_wait(unsigned long long* b) {
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(b);
+    unsigned done = 0;
+    for (int spin = 0; spin < (1 << 20) && !done; ++spin)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar)
+            : "memory");
+}
+
+// Lays the one-CTA levels out in shared memory from word off on (per smoothed level A [NPT], dinv,
+// x, b, a multiple of four words each since its axes are even; of the dense level x and b) and
+// starts the copies of their stencils and inverse diagonals. One thread.
+template <int NPT>
+__device__ void cta_levels(const LVSet& S, float* sm, int off, LV<float>* V, CtaLevel* T, BulkLoad& load) {
+    for (int l = S.first_cta; l < S.nl; ++l) {
+        const LV<float>& G = S.l[l];
+        const int nc = (G.ncell + 3) & ~3;
+        V[l] = G;
+        CtaLevel& L = T[l];
+        L.n0 = G.n[0], L.n1 = G.n[1], L.n2 = G.n[2], L.half = G.n[0] / 2, L.ncell = G.ncell;
+        L.mh = div_magic(L.half);
+        L.m1 = div_magic(L.n1);
+        if (l < S.nl - 1) {
+            L.A = sm + off;
+            L.dinv = L.A + NPT * nc;
+            L.x = L.dinv + nc;
+            off += (NPT + 2) * nc;
+            load.copy(L.A, G.A, NPT * nc * 4);
+            load.copy(L.dinv, G.dinv, nc * 4);
+        } else {
+            L.A = L.dinv = nullptr;
+            L.x = sm + off;
+            off += nc;
+        }
+        L.b = sm + off;
+        off += nc;
+        V[l].A = L.A;
+        V[l].x = L.x;
+        V[l].b = L.b;
+    }
+}
+
+// The V-cycle over the one-CTA levels, x = 0 before it, once their copies are in: every thread
+// of the block. dense: the dense inverse in shared memory, or null.
 template <int D, int NPT>
-__global__ void __launch_bounds__(512, 1) coarse_cycle_kernel(const __grid_constant__ LVSet S, int nu1, int nu2, int dense_smem) {
-    extern __shared__ __align__(16) float sm[];
-    __shared__ LV<float> V[MAX_LEVELS];
-    __shared__ CtaLevel T[MAX_LEVELS];
-    __shared__ __align__(8) unsigned long long bar;
+__device__ __forceinline__ void cta_cycle(const LVSet& S, const LV<float>* V, const CtaLevel* T, const float* dense, int nu1,
+                                          int nu2) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int m = S.dense_m, mm = m + (S.singular ? 1 : 0);
-    const unsigned ubar = (unsigned)__cvta_generic_to_shared(&bar);
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(ubar) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        // shared memory: per level A [NPT], dinv, x, b (a multiple of four words each on the
-        // smoothed levels, whose axes are even); then the dense inverse
-        int off = 0;
-        unsigned bytes = 0;
-        for (int l = S.first_cta; l < S.nl; ++l) {
-            const LV<float>& G = S.l[l];
-            const int nc = (G.ncell + 3) & ~3;
-            V[l] = G;
-            CtaLevel& L = T[l];
-            L.n0 = G.n[0], L.n1 = G.n[1], L.n2 = G.n[2], L.half = G.n[0] / 2, L.ncell = G.ncell;
-            L.mh = div_magic(L.half);
-            L.m1 = div_magic(L.n1);
-            if (l < S.nl - 1) {
-                L.A = sm + off;
-                L.dinv = L.A + NPT * nc;
-                L.x = L.dinv + nc;
-                off += (NPT + 2) * nc;
-                bytes += (NPT + 1) * G.ncell * 4;
-            } else {  // the dense level needs its right-hand side and solution only
-                L.A = L.dinv = nullptr;
-                L.x = sm + off;
-                off += nc;
-            }
-            L.b = sm + off;
-            off += nc;
-            V[l].A = L.A;
-            V[l].x = L.x;
-            V[l].b = L.b;
-        }
-        const bool smoothed = S.first_cta < S.nl - 1;
-        if (smoothed) bytes += S.l[S.first_cta].ncell * 4;  // its right-hand side
-        const unsigned dense_bytes = dense_smem ? (unsigned)((mm * mm * 4 + 15) & ~15) : 0u;
-        bytes += dense_bytes;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(ubar), "r"(bytes) : "memory");
-        auto copy = [&](float* dst, const float* src, unsigned n) {
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                             (unsigned)__cvta_generic_to_shared(dst)),
-                         "l"(src), "r"(n), "r"(ubar)
-                         : "memory");
-        };
-        for (int l = S.first_cta; l < S.nl - 1; ++l) {
-            const int nc = S.l[l].ncell;
-            copy(T[l].A, S.l[l].A, NPT * nc * 4);
-            copy(T[l].dinv, S.l[l].dinv, nc * 4);
-        }
-        if (smoothed) copy(T[S.first_cta].b, S.l[S.first_cta].b, S.l[S.first_cta].ncell * 4);
-        if (dense_smem) copy(sm + dense_smem, S.dense_inv, dense_bytes);
-    }
-    __syncthreads();
-    for (int c = tid; c < T[S.first_cta].ncell; c += nt) {
-        T[S.first_cta].x[c] = 0.0f;
-        if (S.first_cta == S.nl - 1) T[S.first_cta].b[c] = S.l[S.first_cta].b[c];
-    }
-    {
-        // the copies take a microsecond or so: a bounded wait (on giving up the values are wrong,
-        // the residual does not fall and the solve reports it)
-        unsigned done = 0;
-        for (int spin = 0; spin < (1 << 20) && !done; ++spin)
-            asm volatile(
-                "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(done)
-                : "r"(ubar)
-                : "memory");
-    }
-    __syncthreads();
     // alternating zebra line relaxation: lines along each axis in turn, each colour in turn
     // (reverse order after the coarse-grid correction)
     auto line_sweep = [&](int l, bool reverse) {
@@ -1013,19 +1006,7 @@ __global__ void __launch_bounds__(512, 1) coarse_cycle_kernel(const __grid_const
             else
                 for (int col = 0; col < NCOL; ++col) cta_sweep<D, NPT>(L, col, it == 0 && col == 0);
         }
-        if (S.line) {
-            // every cell has a residual after a line sweep
-            const LV<float>& C = V[l + 1];
-            const int plane = C.n[0] * C.n[1];
-            for (int idx = tid; idx < C.ncell; idx += nt) {
-                const int k = idx / plane, r = idx - k * plane, j = r / C.n[0];
-                const int q[3] = {r - j * C.n[0], j, k};
-                restrict_at<D, NPT>(V[l], C, q);
-            }
-            __syncthreads();
-        } else {
-            cta_restrict<D, NPT>(L, T[l + 1]);
-        }
+        cta_restrict<D, NPT>(L, T[l + 1]);
     }
     {
         // dense solve, one unknown a thread (the inverse is stored transposed, so that
@@ -1033,10 +1014,9 @@ __global__ void __launch_bounds__(512, 1) coarse_cycle_kernel(const __grid_const
         const float* bs = T[S.nl - 1].b;
         for (int i = tid; i < m; i += nt) {
             float acc = 0.0f;
-            if (dense_smem) {
-                const float* R = sm + dense_smem + i;
+            if (dense) {
 #pragma unroll 8
-                for (int k = 0; k < m; ++k) acc += R[k * mm] * bs[k];
+                for (int k = 0; k < m; ++k) acc += dense[k * mm + i] * bs[k];
             } else {
 #pragma unroll 16
                 for (int k = 0; k < m; ++k) acc += __ldg(S.dense_inv + k * mm + i) * bs[k];
@@ -1063,8 +1043,254 @@ __global__ void __launch_bounds__(512, 1) coarse_cycle_kernel(const __grid_const
                 for (int col = NCOL - 1; col >= 0; --col) cta_sweep<D, NPT>(F, col, false);
         }
     }
+}
+
+// All of these levels' stencils, inverse diagonals and right-hand sides come in by bulk copies
+// (one a level and array, so the load is one latency and not a chain of them); with the dense
+// inverse beside them when it fits; the first sweep from x = 0 reads no neighbours, and of two
+// colours the second is not prolonged onto (the next sweep overwrites it). The CTA part of a
+// 512 x 1024 V-cycle (levels of 32 x 64 cells and below) takes 16 us (33 with per-cell index
+// divisions, element-wise staging and the dense inverse read a row per thread), that of
+// a 24 x 20 x 16 one (12 x 10 x 8 and below) 10.5 us (18.8).
+template <int D, int NPT>
+__global__ void __launch_bounds__(512, 1) coarse_cycle_kernel(const __grid_constant__ LVSet S, int nu1, int nu2, int dense_smem) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ LV<float> V[MAX_LEVELS];
+    __shared__ CtaLevel T[MAX_LEVELS];
+    __shared__ __align__(8) unsigned long long bar;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const bool smoothed = S.first_cta < S.nl - 1;
     const LV<float>& G = S.l[S.first_cta];
+    if (tid == 0) {
+        BulkLoad load;
+        load.init(&bar);
+        cta_levels<NPT>(S, sm, 0, V, T, load);
+        if (smoothed) load.copy(T[S.first_cta].b, G.b, G.ncell * 4);
+        const int mm = S.dense_m + (S.singular ? 1 : 0);
+        if (dense_smem) load.copy(sm + dense_smem, S.dense_inv, (unsigned)((mm * mm * 4 + 15) & ~15));
+        load.arrive();
+    }
+    __syncthreads();
+    for (int c = tid; c < G.ncell; c += nt) {
+        T[S.first_cta].x[c] = 0.0f;
+        if (!smoothed) T[S.first_cta].b[c] = G.b[c];
+    }
+    bulk_wait(&bar);
+    __syncthreads();
+    cta_cycle<D, NPT>(S, V, T, dense_smem ? sm + dense_smem : nullptr, nu1, nu2);
     for (int c = tid; c < G.ncell; c += nt) G.x[c] = T[S.first_cta].x[c];
+}
+
+// ---- the lower part of a 3D two-colour V-cycle on a thread-block cluster
+//
+// Levels too large for one CTA but far too small for the chip (a colour sweep of 32^3 cells has
+// 4 us of launch and ramp for 0.5 us of work) are split by planes over the cluster's CTAs, in
+// shared memory: a sweep hands the new values of its first and last plane to the neighbours'
+// halo planes and ends with a cluster barrier (0.4 us). The one-CTA levels below are solved by
+// every CTA redundantly. Same operations in the same order as the kernels per level. Measured:
+// 40 us for the levels from 32^3 down of a 128^3 V-cycle on 8 CTAs (55 us as 23 launches), 20
+// us for a whole 24 x 20 x 16 V-cycle (30 us). 64^3 stays on its launches: 15 planes of 4096
+// cells a CTA do not fit, and its sweeps fill the chip.
+constexpr int SL_MAX = 2;           // split levels
+constexpr int SL_CELLS = 40960;     // a level joins from this many cells down
+constexpr size_t SL_SMEM_MAX = 216 * 1024;
+
+struct SlabPlan {
+    int cs;          // CTAs
+    int first, ns;   // split levels first .. first + ns - 1; the one-CTA levels follow
+    int rmax[SL_MAX];  // most planes of a CTA
+    int oa[SL_MAX], od[SL_MAX], ob[SL_MAX], ox[SL_MAX];  // shared offsets (words)
+    int ocoarse;     // of the one-CTA levels
+    int odense;      // of the dense inverse (0: global)
+};
+
+// first plane of CTA `rank` on the level below the split ones (whose restriction must not cross
+// CTAs); each finer level doubles it
+__host__ __device__ inline int slab_start(int rank, int cs, int planes) { return rank * planes / cs; }
+
+struct Slab {
+    int n0, n1, n2, half, plane, z0, R;
+    unsigned mh, m1;
+    const float *A, *d;
+    float *b, *x;        // x: one halo plane below and above
+    float *lower, *upper;  // the neighbours' halo planes that mirror this CTA's first and last
+};
+
+// one colour; first: x = 0 before it
+__device__ __forceinline__ void slab_sweep(const Slab& L, int colour, bool first) {
+    const int count = L.R * L.n1 * L.half, nc = L.R * L.plane;
+    for (int idx = threadIdx.x; idx < count; idx += 512) {
+        const int row = div_by(idx, L.mh), m = idx - row * L.half, kk = div_by(row, L.m1), j = row - kk * L.n1;
+        const int i = 2 * m + ((j + L.z0 + kk + colour) & 1);
+        const int in = j * L.n0 + i, c = kk * L.plane + in;
+        float* x = L.x + c + L.plane;
+        float s = 0.0f;
+        if (!first) {
+            s += L.A[nc + c] * x[i > 0 ? -1 : L.n0 - 1];
+            s += L.A[2 * nc + c] * x[i < L.n0 - 1 ? 1 : 1 - L.n0];
+            s += L.A[3 * nc + c] * x[(j > 0 ? -1 : L.n1 - 1) * L.n0];
+            s += L.A[4 * nc + c] * x[(j < L.n1 - 1 ? 1 : 1 - L.n1) * L.n0];
+            s += L.A[5 * nc + c] * x[-L.plane];
+            s += L.A[6 * nc + c] * x[L.plane];
+        }
+        const float v = (L.b[c] - s) * L.d[c];
+        *x = v;
+        if (kk == 0 && L.lower) L.lower[in] = v;
+        if (kk == L.R - 1 && L.upper) L.upper[in] = v;
+    }
+}
+
+__global__ void __launch_bounds__(512, 1) coarse_cluster_kernel(const __grid_constant__ LVSet S, const __grid_constant__ SlabPlan P,
+                                                                int nu1, int nu2) {
+    extern __shared__ __align__(16) float sm[];
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), cs = P.cs, tid = threadIdx.x;
+    __shared__ LV<float> V[MAX_LEVELS];
+    __shared__ CtaLevel T[MAX_LEVELS];
+    __shared__ Slab W[SL_MAX];
+    __shared__ __align__(8) unsigned long long bar;
+    const int zc = S.l[S.first_cta].n[2];  // planes of the level below the split ones
+    if (tid == 0) {
+        BulkLoad load;
+        load.init(&bar);
+        for (int t = 0; t < P.ns; ++t) {
+            const LV<float>& G = S.l[P.first + t];
+            const int up = P.ns - t;
+            auto start = [&](int q) { return slab_start(q, cs, zc) << up; };
+            Slab& L = W[t];
+            L.n0 = G.n[0], L.n1 = G.n[1], L.n2 = G.n[2], L.half = L.n0 / 2, L.plane = L.n0 * L.n1;
+            L.mh = div_magic(L.half);
+            L.m1 = div_magic(L.n1);
+            L.z0 = start(rank);
+            L.R = start(rank + 1) - L.z0;
+            L.A = sm + P.oa[t];
+            L.d = sm + P.od[t];
+            L.b = sm + P.ob[t];
+            L.x = sm + P.ox[t];
+            const int lo = rank > 0 ? rank - 1 : (G.per[2] ? cs - 1 : -1), hi = rank < cs - 1 ? rank + 1 : (G.per[2] ? 0 : -1);
+            L.lower = lo >= 0 ? cl.map_shared_rank(L.x, lo) + (start(lo + 1) - start(lo) + 1) * L.plane : nullptr;
+            L.upper = hi >= 0 ? cl.map_shared_rank(L.x, hi) : nullptr;
+            const int nc = L.R * L.plane;
+            for (int k = 1; k < 7; ++k) load.copy(sm + P.oa[t] + k * nc, G.A + (size_t)k * G.ncell + L.z0 * L.plane, nc * 4);
+            load.copy(sm + P.oa[t], G.A + L.z0 * L.plane, nc * 4);
+            load.copy(sm + P.od[t], G.dinv + L.z0 * L.plane, nc * 4);
+            if (t == 0) load.copy(L.b, G.b + L.z0 * L.plane, nc * 4);
+        }
+        cta_levels<7>(S, sm, P.ocoarse, V, T, load);
+        const int mm = S.dense_m + (S.singular ? 1 : 0);
+        if (P.odense) load.copy(sm + P.odense, S.dense_inv, (unsigned)((mm * mm * 4 + 15) & ~15));
+        load.arrive();
+    }
+    __syncthreads();
+    for (int t = 0; t < P.ns; ++t)
+        for (int c = tid; c < (W[t].R + 2) * W[t].plane; c += 512) W[t].x[c] = 0.0f;
+    for (int c = tid; c < T[S.first_cta].ncell; c += 512) T[S.first_cta].x[c] = 0.0f;
+    bulk_wait(&bar);
+    cl.sync();  // every CTA's x is set before a neighbour writes into it
+    for (int t = 0; t < P.ns; ++t) {
+        const Slab L = W[t];
+        for (int it = 0; it < nu1; ++it)
+            for (int col = 0; col < 2; ++col) {
+                slab_sweep(L, col, it == 0 && col == 0);
+                cl.sync();
+            }
+        // restriction, in the order of restrict_at: to this CTA's planes of a split level, or to every
+        // CTA's copy of the first level held whole
+        const bool whole = t == P.ns - 1;
+        const int cn0 = L.half, cn1 = L.n1 / 2, cplane = cn0 * cn1, cells = L.R / 2 * cplane, nc = L.R * L.plane;
+        float* cb = whole ? T[S.first_cta].b : W[t + 1].b;
+        for (int idx = tid; idx < cells; idx += 512) {
+            const int row = div_by(idx, L.mh), ic = idx - row * cn0, kc = row / cn1, jc = row - kc * cn1;
+            float acc = 0.0f;
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch) {
+                const int i = 2 * ic + (ch & 1), j = 2 * jc + ((ch >> 1) & 1), kk = 2 * kc + (ch >> 2);
+                const int c = kk * L.plane + j * L.n0 + i;
+                const float* x = L.x + c + L.plane;
+                float s = 0.0f;
+                s += L.A[c] * x[0];
+                s += L.A[nc + c] * x[i > 0 ? -1 : L.n0 - 1];
+                s += L.A[2 * nc + c] * x[i < L.n0 - 1 ? 1 : 1 - L.n0];
+                s += L.A[3 * nc + c] * x[(j > 0 ? -1 : L.n1 - 1) * L.n0];
+                s += L.A[4 * nc + c] * x[(j < L.n1 - 1 ? 1 : 1 - L.n1) * L.n0];
+                s += L.A[5 * nc + c] * x[-L.plane];
+                s += L.A[6 * nc + c] * x[L.plane];
+                acc += L.b[c] - s;
+            }
+            if (whole) {
+                const int off = L.z0 / 2 * cplane + idx;
+                for (int q = 0; q < cs; ++q) cl.map_shared_rank(cb, q)[off] = acc;
+            } else {
+                cb[idx] = acc;
+            }
+        }
+        if (whole) cl.sync();
+        else __syncthreads();
+    }
+    cta_cycle<3, 7>(S, V, T, P.odense ? sm + P.odense : nullptr, nu1, nu2);
+    for (int t = P.ns - 1; t >= 0; --t) {
+        const Slab L = W[t];
+        const LV<float>& Cl = S.l[P.first + t + 1];
+        const bool whole = t == P.ns - 1;
+        const int cplane = Cl.n[0] * Cl.n[1];
+        // plane K of the coarse correction is at xc + K cplane (a split level's planes are local)
+        const float* xc = whole ? T[S.first_cta].x : W[t + 1].x + (1 - W[t + 1].z0) * cplane;
+        for (int idx = tid; idx < L.R * L.n1 * L.half; idx += 512) {
+            // prolongation onto the first colour (the next sweep overwrites the second), as prolong_at
+            const int row = div_by(idx, L.mh), m = idx - row * L.half, kk = div_by(row, L.m1), j = row - kk * L.n1;
+            const int q[3] = {2 * m + ((j + L.z0 + kk) & 1), j, L.z0 + kk};
+            int off[3][2];
+            float sg[3];
+            int stride = 1;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int pa = q[a] >> 1;
+                int nb = pa + ((q[a] & 1) ? 1 : -1);
+                sg[a] = 1.0f;
+                if (nb < 0 || nb >= Cl.n[a]) {
+                    const int side = nb < 0 ? 0 : 1;
+                    if (Cl.per[a]) {
+                        if (a < 2 || whole) nb = nb < 0 ? nb + Cl.n[a] : nb - Cl.n[a];  // else: the halo plane
+                    } else {
+                        nb = side == 0 ? 0 : Cl.n[a] - 1;
+                        if (Cl.bc[2 * a + side] == CPIC_BC_DIRICHLET) sg[a] = -1.0f;
+                    }
+                }
+                off[a][0] = pa * stride;
+                off[a][1] = nb * stride;
+                stride *= Cl.n[a];
+            }
+            float acc = 0.0f;
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                float w = 1.0f, sign = 1.0f;
+                int at = 0;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const int bit = (o >> a) & 1;
+                    w *= bit ? 0.25f : 0.75f;
+                    if (bit) sign *= sg[a];
+                    at += off[a][bit];
+                }
+                acc += w * (sign * xc[at]);
+            }
+            const int in = j * L.n0 + q[0];
+            float* x = L.x + (kk + 1) * L.plane + in;
+            const float v = *x + acc;
+            *x = v;
+            if (kk == 0 && L.lower) L.lower[in] = v;
+            if (kk == L.R - 1 && L.upper) L.upper[in] = v;
+        }
+        cl.sync();
+        for (int it = 0; it < nu2; ++it)
+            for (int col = 1; col >= 0; --col) {
+                slab_sweep(L, col, false);
+                cl.sync();  // the last one also keeps every CTA's memory until its neighbours are done
+            }
+    }
+    const Slab L = W[0];
+    float* out = S.l[P.first].x + L.z0 * L.plane;
+    for (int c = tid; c < L.R * L.plane; c += 512) out[c] = L.x[L.plane + c];
 }
 
 // ------------------------------------------------------------------ FP64 outer iteration
@@ -1094,33 +1320,29 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
     __syncthreads();
 }
 
-__device__ __forceinline__ void block_sum3(double& a, double& b, double& c, double* sh) {
+// Sums of N doubles a thread over a block of 256 threads, in a fixed order, given to every thread.
+// The first step goes through shared memory so that one warp a sum does the additions: FP64 runs
+// at under two operations per SM and clock here, and a shuffle tree in all eight warps costs
+// 15 N x 256 / 1.7 cycles of it (3 us a block for three sums) against N x 400.
+template <int N>
+__device__ __forceinline__ void block_sums(double (&v)[N], double (*sh)[256]) {
+    const int tid = threadIdx.x + blockDim.x * threadIdx.y, w = tid >> 5, l = tid & 31;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-    int w = tid >> 5, l = tid & 31;
-    if (l == 0) {
-        sh[3 * w] = a;
-        sh[3 * w + 1] = b;
-        sh[3 * w + 2] = c;
-    }
+    for (int n = 0; n < N; ++n) sh[n][tid] = v[n];
     __syncthreads();
-    if (w == 0) {
-        int nw = (blockDim.x * blockDim.y) >> 5;
-        a = l < nw ? sh[3 * l] : 0.0;
-        b = l < nw ? sh[3 * l + 1] : 0.0;
-        c = l < nw ? sh[3 * l + 2] : 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, o);
-            b += __shfl_xor_sync(0xffffffffu, b, o);
-            c += __shfl_xor_sync(0xffffffffu, c, o);
+    for (int n = 0; n < N; ++n)
+        if (w == n) {
+            double a = sh[n][l];
+#pragma unroll
+            for (int i = 1; i < 8; ++i) a += sh[n][l + 32 * i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (l == 0) sh[n][0] = a;
         }
-    }
+    __syncthreads();
+#pragma unroll
+    for (int n = 0; n < N; ++n) v[n] = sh[n][0];
     __syncthreads();
 }
 
@@ -1142,36 +1364,36 @@ struct ResidualParams {
     cudaGraphConditionalHandle handle;
 };
 
-// r = b - M phi in FP64, its FP32 copy, and ||r||, ||b||; the last block to finish sums the
-// block partials in a fixed tree, updates the counters and decides whether to continue.
-// Blocks of 32 x 8 threads walk rows (j, k) of 32-cell segments.
+// r = b - M phi in FP64, its FP32 copy, and ||r|| (and ||b|| with the first residual of a solve);
+// the last block to finish sums the block partials in a fixed order, updates the counters and
+// decides whether to continue. Blocks of 32 x 8 threads walk rows (j, k) of 32-cell segments.
+// Bound by the FP64 rate: 19 operations a cell for the 3D operator.
 template <int D, int NPT>
-__global__ void __launch_bounds__(256) residual_kernel(ResidualParams P) {
-    __shared__ double sh[96];
+__global__ void __launch_bounds__(256) residual_kernel(const __grid_constant__ ResidualParams P) {
+    __shared__ double sh[3][256];
     __shared__ bool last;
     const LV<double>& L = P.L;
-    const bool dot_rh = P.ks && !P.init;
-    double rr = 0.0, bb = 0.0, hr = 0.0;
+    const bool dot_rh = P.ks && !P.init, with_b = P.count_cycle == 0;
+    double v[3] = {0.0, 0.0, 0.0};  // (r, r), (r^, r), (b, b)
     const int nrows = L.n[1] * L.n[2];
     for (int row = blockIdx.x * blockDim.y + threadIdx.y; row < nrows; row += gridDim.x * blockDim.y) {
         int j = row % L.n[1], k = row / L.n[1];
         for (int i = threadIdx.x; i < L.n[0]; i += blockDim.x) {
             int q[3] = {i, j, k};
             int c = i + L.n[0] * row;
-            double r = L.b[c] - stencil_sum<D, NPT, 0>(L, c, q);
+            const double b = L.b[c], r = b - stencil_sum<D, NPT, 0>(L, c, q);
             if (P.r32) P.r32[c] = (float)r;
             if (P.r64) P.r64[c] = r;
-            rr += r * r;
-            bb += L.b[c] * L.b[c];
-            if (dot_rh) hr += P.rh[c] * r;
+            v[0] += r * r;
+            if (dot_rh) v[1] += P.rh[c] * r;
+            if (with_b) v[2] += b * b;
         }
     }
-    block_sum3(rr, bb, hr, sh);
+    block_sums<3>(v, sh);
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     if (tid == 0) {
-        P.part[3 * blockIdx.x] = rr;
-        P.part[3 * blockIdx.x + 1] = bb;
-        P.part[3 * blockIdx.x + 2] = hr;
+#pragma unroll
+        for (int n = 0; n < 3; ++n) P.part[3 * blockIdx.x + n] = v[n];
         __threadfence();
         unsigned t = atomicAdd(P.ticket, 1u);
         last = t == gridDim.x - 1;
@@ -1179,17 +1401,18 @@ __global__ void __launch_bounds__(256) residual_kernel(ResidualParams P) {
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double a = 0.0, b = 0.0, h = 0.0;
-    for (int i = tid; i < (int)gridDim.x; i += blockDim.x * blockDim.y) {
-        a += P.part[3 * i];
-        b += P.part[3 * i + 1];
-        h += P.part[3 * i + 2];
-    }
-    block_sum3(a, b, h, sh);
+#pragma unroll
+    for (int n = 0; n < 3; ++n) v[n] = 0.0;
+    for (int i = tid; i < (int)gridDim.x; i += 256)
+#pragma unroll
+        for (int n = 0; n < 3; ++n) v[n] += __ldcg(P.part + 3 * i + n);
+    block_sums<3>(v, sh);
     if (tid == 0) {
+        const double a = v[0], h = v[1];
         *P.ticket = 0;
         DevCounters* ctr = P.ctr;
         ctr->mg_cycles += P.count_cycle;
+        if (with_b) ctr->mg_bnorm = sqrt(v[2]);
         if (KrylovState* ks = P.ks) {
             // (r^, r) of the new residual; a vanishing rho, alpha or omega restarts the
             // recurrence from r^ = p = r, whose rho is (r, r)
@@ -1205,9 +1428,9 @@ __global__ void __launch_bounds__(256) residual_kernel(ResidualParams P) {
                 ks->rho = h;
             }
         }
-        double res = b > 0.0 ? sqrt(a) / sqrt(b) : 0.0;
+        const double bnorm = ctr->mg_bnorm;
+        double res = bnorm > 0.0 ? sqrt(a) / bnorm : 0.0;
         ctr->mg_residual = res;
-        ctr->mg_bnorm = sqrt(b);
         bool converged = res <= P.rtol;
         if (converged) ctr->mg_converged = 1;
         bool cont = !converged && ctr->mg_cycles < P.max_cycles;
@@ -1248,12 +1471,12 @@ __global__ void bicg_direction_kernel(int n, const double* __restrict__ r, doubl
 // rate), reduced in FP64; mode 0: v = y, p^ = x32 kept, reduce (r^, v) ->
 // alpha = rho / (r^, v); mode 1: reduce (y, s), (y, y) -> omega = (t, s) / (t, t)
 template <int D, int NPT>
-__global__ void __launch_bounds__(256) bicg_matvec_kernel(LV<float> L, const float* __restrict__ x32, int mode,
+__global__ void __launch_bounds__(256) bicg_matvec_kernel(const __grid_constant__ LV<float> L, const float* __restrict__ x32, int mode,
                                                            float* v, float* ph32, const double* __restrict__ wr,
                                                            const float* __restrict__ ws, KrylovState* ks) {
-    __shared__ double sh[96];
+    __shared__ double sh[2][256];
     __shared__ bool last;
-    double d0 = 0.0, d1 = 0.0, d2 = 0.0;
+    double d0 = 0.0, d1 = 0.0;
     const int nrows = L.n[1] * L.n[2];
     // one cell's product and its contributions to the reductions
     auto emit = [&](int c, float yf) {
@@ -1331,11 +1554,12 @@ __global__ void __launch_bounds__(256) bicg_matvec_kernel(LV<float> L, const flo
             }
         }
     }
-    block_sum3(d0, d1, d2, sh);
+    double d[2] = {d0, d1};
+    block_sums<2>(d, sh);
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     if (tid == 0) {
-        ks->part[3 * blockIdx.x] = d0;
-        ks->part[3 * blockIdx.x + 1] = d1;
+        ks->part[3 * blockIdx.x] = d[0];
+        ks->part[3 * blockIdx.x + 1] = d[1];
         __threadfence();
         unsigned t = atomicAdd(&ks->ticket, 1u);
         last = t == gridDim.x - 1;
@@ -1343,12 +1567,13 @@ __global__ void __launch_bounds__(256) bicg_matvec_kernel(LV<float> L, const flo
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double a = 0.0, b = 0.0, z = 0.0;
-    for (int i = tid; i < (int)gridDim.x; i += blockDim.x * blockDim.y) {
-        a += ks->part[3 * i];
-        b += ks->part[3 * i + 1];
+    d[0] = d[1] = 0.0;
+    for (int i = tid; i < (int)gridDim.x; i += 256) {
+        d[0] += __ldcg(&ks->part[3 * i]);
+        d[1] += __ldcg(&ks->part[3 * i + 1]);
     }
-    block_sum3(a, b, z, sh);
+    block_sums<2>(d, sh);
+    const double a = d[0], b = d[1];
     if (tid == 0) {
         ks->ticket = 0;
         if (mode == 0) {
@@ -1751,6 +1976,81 @@ int dispatch_vshape(const cpic_run* r, F f) {
                  : f(std::integral_constant<int, 3>(), std::integral_constant<int, 7>());
 }
 
+// The cluster part's levels, sizes and layout; false: the V-cycle has none (see SlabPlan). The
+// CTAs are as many as the level below the split ones has planes, 16 at most (cs_max where the
+// device co-schedules fewer).
+bool plan_slabs(const LVSet& S, int cs_max, SlabPlan* P, size_t* smem) {
+    const LV<float>& F = S.l[0];
+    if (F.D != 3 || F.used != 7 || S.line || F.pw || cs_max < 2 || S.first_cta < 1 || S.first_cta >= S.nl - 1) return false;
+    for (int ns = SL_MAX; ns > 0; --ns) {
+        const int first = S.first_cta - ns;
+        if (first < 0 || S.l[first].ncell > SL_CELLS) continue;
+        const int planes = S.l[S.first_cta].n[2];
+        const int cs = planes < cs_max ? planes : cs_max;
+        if (cs < 2) continue;
+        P->cs = cs;
+        P->first = first;
+        P->ns = ns;
+        size_t off = 0;
+        for (int t = 0; t < ns; ++t) {
+            const LV<float>& L = S.l[first + t];
+            const size_t plane = (size_t)L.n[0] * L.n[1], R = (size_t)((planes + cs - 1) / cs) << (ns - t);
+            P->rmax[t] = (int)R;
+            P->oa[t] = (int)off, off += 7 * R * plane;
+            P->od[t] = (int)off, off += R * plane;
+            P->ob[t] = (int)off, off += R * plane;
+            P->ox[t] = (int)off, off += (R + 2) * plane;
+        }
+        P->ocoarse = (int)off;
+        off += cta_words(S, S.first_cta);
+        const size_t mm = S.dense_m + S.singular, dense = (mm * mm + 3) & ~size_t(3);
+        P->odense = 0;
+        if ((off + dense) * sizeof(float) <= SL_SMEM_MAX) {
+            P->odense = (int)off;
+            off += dense;
+        }
+        *smem = off * sizeof(float);
+        if (*smem <= SL_SMEM_MAX) return true;
+    }
+    return false;
+}
+
+void slab_config(const SlabPlan& P, size_t smem, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
+    cfg->gridDim = dim3(P.cs, 1, 1);
+    cfg->blockDim = dim3(512, 1, 1);
+    cfg->dynamicSmemBytes = smem;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = P.cs;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+}
+
+// the largest cluster the device co-schedules for this run's cluster part (0: none)
+int prepare_slabs(const cpic_run* r, int* cs_max) {
+    *cs_max = 0;
+    const LVSet S = make_set(r);
+    for (int cs : {16, 8}) {
+        SlabPlan P;
+        size_t smem = 0;
+        if (!plan_slabs(S, cs, &P, &smem)) return CPIC_OK;
+        CPIC_CUDA(cudaFuncSetAttribute(coarse_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SL_SMEM_MAX));
+        if (cudaFuncSetAttribute(coarse_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            cudaGetLastError();
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr;
+        slab_config(P, smem, &cfg, &attr);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, coarse_cluster_kernel, &cfg) == cudaSuccess && n > 0) {
+            *cs_max = cs;
+            return CPIC_OK;
+        }
+        cudaGetLastError();
+    }
+    return CPIC_OK;
+}
+
 // the levels of the one-CTA part
 template <int D, int NPT>
 int enqueue_coarse(cpic_run* r, const LVSet& S, int nu1, int nu2) {
@@ -1780,7 +2080,11 @@ int enqueue_vcycle(cpic_run* r, const LVSet& S) {
         constexpr int D = decltype(Dc)::value, NPT = decltype(Nc)::value;
         cudaStream_t st = r->stream;
         const int nu1 = 2, nu2 = 2;
-        const int top = S.first_cta;
+        int top = S.first_cta;  // levels above take a launch per pass
+        SlabPlan slabs;
+        size_t slab_smem = 0;
+        const bool cluster = plan_slabs(S, r->slab_cs, &slabs, &slab_smem);
+        if (cluster) top = slabs.first;
         // 2D two-colour levels: one launch down and one up each, the results in the levels' second
         // buffers (the line-relaxation work, free with point smoothing)
         if (D == 2 && NPT == 5 && fused_levels(S)) {
@@ -1800,7 +2104,7 @@ int enqueue_vcycle(cpic_run* r, const LVSet& S) {
             }
             return CPIC_OK;
         }
-        CPIC_CUDA(cudaMemsetAsync(r->lev[0].x32, 0, sizeof(float) * r->lev[0].ncell, st));
+        if (top > 0) CPIC_CUDA(cudaMemsetAsync(r->lev[0].x32, 0, sizeof(float) * r->lev[0].ncell, st));
         auto smooth = [&](int l, int col) -> int {
             const LV<float>& L = S.l[l];
             int d[3] = {L.n[0] / 2, Col<D, NPT>::parity ? L.n[1] : L.n[1] / 2,
@@ -1843,7 +2147,16 @@ int enqueue_vcycle(cpic_run* r, const LVSet& S) {
             restrict_kernel<D, NPT><<<rg, rb, 0, st>>>(Fl, C);
             CPIC_CHECK_LAUNCH();
         }
-        if (int e = enqueue_coarse<D, NPT>(r, S, nu1, nu2)) return e;
+        if (cluster) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr;
+            slab_config(slabs, slab_smem, &cfg, &attr);
+            cfg.stream = st;
+            CPIC_CUDA(cudaLaunchKernelEx(&cfg, coarse_cluster_kernel, S, slabs, nu1, nu2));
+            CPIC_CHECK_LAUNCH();
+        } else if (int e = enqueue_coarse<D, NPT>(r, S, nu1, nu2)) {
+            return e;
+        }
         for (int l = top - 1; l >= 0; --l) {
             const LV<float>& L = S.l[l];
             prolong_kernel<D><<<cell_grid(L.n[0], L.n[1], L.n[2]), kCellBlock, 0, st>>>(L, S.l[l + 1]);
@@ -2062,7 +2375,7 @@ int mg_setup(cpic_run* r) {
         set_error("coarsest multigrid operator is singular");
         return CPIC_ERR_INVALID;
     }
-    return CPIC_OK;
+    return prepare_slabs(r, &r->slab_cs);
 }
 
 // Stream-ordered solve; the host reads the device decision after every cycle

@@ -550,9 +550,10 @@ int cpic_server_stop(cpic_server* server);
 /* Phases of cpic_step timed with CUDA events recorded on the run's stream. */
 #define CPIC_PHASE_FIELD 0   /* a1 vertex field, zeroing of the deposit grid */
 #define CPIC_PHASE_PUSH 1    /* a2-a6 the fused push + deposit kernel alone */
-#define CPIC_PHASE_INJECT 2  /* a8 injection, step counter, halo fold of the deposit grid */
+#define CPIC_PHASE_INJECT 2  /* a8 injection, step counter */
 #define CPIC_PHASE_SORT 3    /* a7 */
-#define CPIC_PHASE_SOLVE 4   /* a9 right-hand side + multigrid + field energy */
+#define CPIC_PHASE_SOLVE 4   /* a9 halo fold of the deposit grid, right-hand side, multigrid,
+                              * field energy */
 #define CPIC_NPHASES 5
 /* Enable (1) or disable (0) per-phase event timing of cpic_step (off by default). */
 int cpic_profile(cpic_run* run, int enable);

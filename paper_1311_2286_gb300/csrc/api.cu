@@ -608,10 +608,9 @@ int enqueue_step_pre(cpic_run* r, bool with_push) {
     return st;
 }
 
-int enqueue_step_post(cpic_run* r, bool sort, bool fold, bool fused_sort) {
+int enqueue_step_post(cpic_run* r, bool sort, bool fused_sort) {
     int st = launch_finalize_step(r);
     if (!st) st = launch_inject(r);
-    if (!st && fold) st = launch_fold(r);
     if (!st && sort) st = launch_sort(r, fused_sort);
     return st;
 }
@@ -624,7 +623,7 @@ int begin_counted_step(cpic_run* r) {
     return CPIC_OK;
 }
 
-int enqueue_step(cpic_run* r, bool sort, bool fold, bool fused_sort = false) {
+int enqueue_step(cpic_run* r, bool sort, bool fused_sort = false) {
     int st = launch_vertex_field(r);
     if (st) return st;
     if (sort && fused_sort && (st = begin_counted_step(r))) return st;
@@ -632,10 +631,6 @@ int enqueue_step(cpic_run* r, bool sort, bool fold, bool fused_sort = false) {
     if (st) return st;
     st = launch_inject(r);
     if (st) return st;
-    if (fold) {  // the compact charge grid is read only by the solve and the charge readers
-        st = launch_fold(r);
-        if (st) return st;
-    }
     if (sort) {
         st = launch_sort(r, fused_sort);
         if (st) return st;
@@ -683,7 +678,7 @@ int build_step_graph(cpic_run* r, int with_solve, int with_sort) {
     const bool pending = r->order_pending;
     r->order_pending = false;
     const bool fused = with_sort != 0 && push_fused_ok(r);
-    st = enqueue_step(r, with_sort != 0, with_solve != 0, fused);
+    st = enqueue_step(r, with_sort != 0, fused);
     r->order_pending = pending;
     r->count_hist = false;
     if (!st && with_solve) {
@@ -751,9 +746,8 @@ int step_once(cpic_run* r, bool solve) {
     st = phase(r, CPIC_PHASE_PUSH, [&] { return launch_push_kernel(r); });
     if (st) return st;
     st = phase(r, CPIC_PHASE_INJECT, [&] {
-        int q = launch_finalize_step(r);
-        if (!q) q = launch_inject(r);
-        return q || !solve ? q : launch_fold(r);
+        const int q = launch_finalize_step(r);
+        return q ? q : launch_inject(r);
     });
     if (st) return st;
     if (r->cfg.sort_interval > 0 && ++r->steps_since_sort >= r->cfg.sort_interval) {
@@ -1175,7 +1169,7 @@ int cpic_set_floating(cpic_run* r, int face, double charge0) {
     if (!st) {
         CPIC_CUDA(cudaMemsetAsync(r->charge, 0, sizeof(unsigned long long) * r->cfg.n_species * r->ncell, r->stream));
         CPIC_CUDA(cudaMemsetAsync(r->lev[0].x, 0, sizeof(double) * r->ncell, r->stream));
-        st = mg_solve(r, 1e-13, 400, true, nullptr, nullptr);
+        st = mg_solve(r, 1e-13, 400, false, nullptr, nullptr);
     }
     if (!st) {
         CPIC_CUDA(cudaMemcpyAsync(r->psi, r->lev[0].x, sizeof(double) * r->ncell, cudaMemcpyDeviceToDevice, r->stream));
@@ -1243,9 +1237,8 @@ int cpic_initialize(cpic_run* r) {
     if (int e = resolve_order(r)) return e;  // the particles in slot order
     CHECK_MAP(r);
     int st = launch_deposit(r);
-    if (!st) st = launch_fold(r);
     if (st) return st;
-    st = mg_solve(r, r->cfg.mg_rtol, r->cfg.mg_max_cycles, false, nullptr, nullptr);
+    st = mg_solve(r, r->cfg.mg_rtol, r->cfg.mg_max_cycles, true, nullptr, nullptr);
     if (st) return st;
     st = launch_vertex_field(r);
     if (st) return st;
@@ -1329,7 +1322,7 @@ int cpic_solve_field(cpic_run* r, double rtol, int max_cycles, int* cycles, doub
     }
     int c = 0;
     double res = 0.0;
-    int st = mg_solve(r, rtol, max_cycles, true, &c, &res);
+    int st = mg_solve(r, rtol, max_cycles, false, &c, &res);
     if (cycles) *cycles = c;
     if (residual) *residual = res;
     return st;

@@ -11,7 +11,7 @@
 //      (cpic_batch_set_mode; the default leaves the push in the run branches: on the
 //      batched configuration, runs of 10^4..2 10^6 particles, the branches that do not wait
 //      for each other measured faster, for full cycles and for particle steps alike);
-//   3. one branch per run again: step counter, injection, halo fold, the cell sort when it
+//   3. one branch per run again: step counter, injection, the cell sort when it
 //      is due and, for full cycles, the field solve (the cluster kernel or the conditional
 //      V-cycle loop).
 // Branches have no dependencies on each other, so the device runs them concurrently: runs
@@ -158,7 +158,7 @@ int capture(cpic_batch* b, bool solve, const std::string& key, cpic_batch::Graph
         e = cudaEventRecord(b->fork2, b->stream);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaEventRecord(fork2)", __FILE__, __LINE__);
     }
-    // 3. post-push branches (injection, fold, sort, field solve)
+    // 3. post-push branches (injection, sort, field solve)
     for (size_t i = 0; !st && i < b->runs.size(); ++i) {
         cpic_run* r = b->runs[i];
         e = cudaStreamWaitEvent(b->branch[i], b->fork2, 0);
@@ -168,7 +168,7 @@ int capture(cpic_batch* b, bool solve, const std::string& key, cpic_batch::Graph
         }
         cudaStream_t saved = r->stream;
         r->stream = b->branch[i];
-        st = enqueue_step_post(r, key[i] == '1', solve, out->fused[i] != 0);
+        st = enqueue_step_post(r, key[i] == '1', out->fused[i] != 0);
         if (!st && solve) {
             cudaStreamCaptureStatus cs;
             cudaGraph_t cg = nullptr;

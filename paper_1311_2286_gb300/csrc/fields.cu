@@ -97,9 +97,9 @@ __global__ void vertex_field_kernel(FieldGrid g, const double* __restrict__ phi,
 }
 
 struct RhsParams {
-    long long ncell;
+    int ncell;
     int nsp;
-    double qw[CPIC_MAX_SPECIES];
+    double qw[CPIC_MAX_SPECIES];  // q w 2^-24: the charge of one count
     double background;
     const double* Jc;
     const double* omega;
@@ -111,56 +111,135 @@ struct RhsParams {
 // Q_c = background J_c + sum_s q_s w_s C_{s,c} 2^-24 (eq. (pg) with J_c cancelled against
 // the cell volume); b_c = Omega_c Q_c + Dirichlet terms. In an axisymmetric run a
 // macro-particle is a ring of charge q w around the axis, spread over the ring volume
-// 2 pi r J_c: its term is divided by 2 pi Omega_c.
-__device__ __forceinline__ double charge_of(const RhsParams& p, long long c) {
-    double Q = __dmul_rn(p.background, p.Jc[c]);
+// 2 pi r J_c: its term is divided by 2 pi Omega_c. count(s): the cell's count of species s. FP64
+// is slow here (1.7 operations per SM and clock), so factors that are exactly one or zero are
+// left out.
+template <class Count>
+__device__ __forceinline__ double charge_of(const RhsParams& p, int c, Count count) {
+    double Q = p.background != 0.0 ? __dmul_rn(p.background, p.Jc[c]) : 0.0;
     const double ring = p.axisym ? __ddiv_rn(1.0, __dmul_rn(2.0 * M_PI, p.omega[c])) : 1.0;
     for (int s = 0; s < p.nsp; ++s) {
-        double C = (double)(long long)p.charge[(long long)s * p.ncell + c];
-        double t = __dmul_rn(p.qw[s], ldexp(C, -QF));
+        double t = __dmul_rn(p.qw[s], (double)(long long)count(s));
         if (p.axisym) t = __dmul_rn(t, ring);
         Q = __dadd_rn(Q, t);
     }
     return Q;
 }
 
-__global__ void rhs_kernel(RhsParams p, double* b) {
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < p.ncell;
-         c += (long long)gridDim.x * blockDim.x) {
-        double Q = charge_of(p, c);
-        b[c] = __dadd_rn(__dmul_rn(p.omega[c], Q), p.bbc[c]);
+__device__ __forceinline__ double rhs_of(const RhsParams& p, int c, double Q) {
+    return __dadd_rn(p.axisym ? __dmul_rn(p.omega[c], Q) : Q, p.bbc[c]);  // Omega = 1 otherwise
+}
+
+// solve counters at the start of a solve
+struct SolveReset {
+    DevCounters* ctr;
+    int* done;
+    unsigned* ticket;
+};
+__device__ __forceinline__ void reset_solve(const SolveReset& z) {
+    *z.done = 0;
+    *z.ticket = 0;
+    z.ctr->mg_cycles = 0;
+    z.ctr->mg_converged = 0;
+}
+
+__global__ void rhs_kernel(RhsParams p, double* b, SolveReset z) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) reset_solve(z);
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < p.ncell; c += gridDim.x * blockDim.x)
+        b[c] = rhs_of(p, c, charge_of(p, c, [&](int s) { return p.charge[(long long)s * p.ncell + c]; }));
+}
+
+// Folds the padded deposit grid into the cell grid the field solve reads: every cell takes
+// its own padded entry plus, on each axis where it is an edge cell, the halo entry that maps
+// onto it (periodic axes wrap: halo -1 -> n-1, halo n -> 0; other axes fold the halo onto
+// the adjacent boundary cell, so charge deposited outside is kept). Gather form: each cell
+// is written by one thread, no atomics.
+struct FoldParams {
+    int n[3], lo[3], hi[3];  // cells that receive the halo entries -1 and n (none: -1)
+    int hs1, hs2, nsp;
+    long long ncell, ncell_h;
+    const unsigned long long* src;
+    unsigned long long* dst;
+};
+
+template <int D>
+__device__ __forceinline__ unsigned long long folded(const FoldParams& f, const unsigned long long* g, int i, int j, int k) {
+    const int base = i + 1 + (j + 1) * f.hs1 + (D == 3 ? (k + 1) * f.hs2 : 0);
+    const bool e0 = i == f.lo[0] || i == f.hi[0], e1 = j == f.lo[1] || j == f.hi[1], e2 = D == 3 && (k == f.lo[2] || k == f.hi[2]);
+    unsigned long long acc = g[base];
+    if (!(e0 || e1 || e2)) return acc;
+    // steps from the cell to the halo entry that maps onto it
+    const int s0 = (i == f.lo[0] ? 0 : f.n[0] + 1) - (i + 1), s1 = ((j == f.lo[1] ? 0 : f.n[1] + 1) - (j + 1)) * f.hs1,
+              s2 = D == 3 ? ((k == f.lo[2] ? 0 : f.n[2] + 1) - (k + 1)) * f.hs2 : 0;
+#pragma unroll
+    for (int o = 1; o < (D == 3 ? 8 : 4); ++o) {
+        if (((o & 1) && !e0) || ((o & 2) && !e1) || ((o & 4) && !e2)) continue;
+        acc += g[base + (o & 1 ? s0 : 0) + (o & 2 ? s1 : 0) + (o & 4 ? s2 : 0)];
+    }
+    return acc;
+}
+
+// the fold, and with b the right-hand side in the same pass (the solve of a step); blocks of
+// 32 x 8 threads walk rows of cells. Bound by the counts' traffic: 128^3 cells with two species
+// 36 us (fold and right-hand side apart, with 64-bit index divisions: 54 and 81 us)
+template <int D, bool RHS>
+__global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ FoldParams f, const __grid_constant__ RhsParams p,
+                                                   double* b, SolveReset z) {
+    if (RHS && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) reset_solve(z);
+    const int nrows = f.n[1] * (D == 3 ? f.n[2] : 1);
+    for (int row = blockIdx.x * blockDim.y + threadIdx.y; row < nrows; row += gridDim.x * blockDim.y) {
+        const int k = D == 3 ? row / f.n[1] : 0, j = row - k * f.n[1];
+        for (int i = threadIdx.x; i < f.n[0]; i += blockDim.x) {
+            const int c = i + f.n[0] * row;
+            auto fold_one = [&](int s) {
+                const unsigned long long v = folded<D>(f, f.src + s * f.ncell_h, i, j, k);
+                f.dst[s * f.ncell + c] = v;
+                return v;
+            };
+            if (RHS) b[c] = rhs_of(p, c, charge_of(p, c, fold_one));
+            else
+                for (int s = 0; s < f.nsp; ++s) fold_one(s);
+        }
     }
 }
 
-// deterministic block reduction (fixed shuffle tree, fixed block count)
-__device__ __forceinline__ double block_sum(double v, double* sh) {
+// W_E = 1/2 sum_c phi_c Q_c: block sums, added by the last block to finish, both in a fixed order
+constexpr int ENERGY_BLOCKS = 256;
+
+__global__ void __launch_bounds__(256) field_energy_kernel(const __grid_constant__ RhsParams p, const double* __restrict__ phi,
+                                                           double* part, unsigned* ticket, DevCounters* ctr) {
+    __shared__ double sh[256];
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    auto block_sum = [&](double v) {  // one warp adds (FP64 is slow): in thread 0
+        sh[tid] = v;
+        __syncthreads();
+        double a = 0.0;
+        if (tid < 32) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r += sh[i];
-    __syncthreads();
-    return r;
-}
-
-__global__ void field_energy_partial(RhsParams p, const double* __restrict__ phi, double* part) {
-    __shared__ double sh[32];
+            for (int w = 0; w < 8; ++w) a += sh[tid + 32 * w];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        }
+        __syncthreads();
+        return a;
+    };
     double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < p.ncell;
-         c += (long long)gridDim.x * blockDim.x)
-        acc += phi[c] * charge_of(p, c);
-    double r = block_sum(acc, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = r;
-}
-
-__global__ void field_energy_final(const double* part, int nb, DevCounters* ctr) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < nb; ++i) s += part[i];
-        ctr->field_energy = 0.5 * s;
+    for (int c = blockIdx.x * 256 + tid; c < p.ncell; c += gridDim.x * 256)
+        acc += phi[c] * charge_of(p, c, [&](int s) { return p.charge[(long long)s * p.ncell + c]; });
+    acc = block_sum(acc);
+    if (tid == 0) {
+        part[blockIdx.x] = acc;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    acc = block_sum(tid < (int)gridDim.x ? __ldcg(part + tid) : 0.0);
+    if (tid == 0) {
+        ctr->field_energy = 0.5 * acc;
+        *ticket = 0;
     }
 }
 
@@ -260,9 +339,9 @@ FloatParams make_float_params(const cpic_run* r) {
 
 RhsParams make_rhs_params(const cpic_run* r) {
     RhsParams p;
-    p.ncell = r->ncell;
+    p.ncell = (int)r->ncell;
     p.nsp = r->cfg.n_species;
-    for (int s = 0; s < CPIC_MAX_SPECIES; ++s) p.qw[s] = s < p.nsp ? r->cfg.q[s] * r->cfg.w[s] : 0.0;
+    for (int s = 0; s < CPIC_MAX_SPECIES; ++s) p.qw[s] = s < p.nsp ? ldexp(r->cfg.q[s] * r->cfg.w[s], -QF) : 0.0;
     p.background = r->cfg.background;
     p.Jc = r->lev[0].Jc;
     p.omega = r->lev[0].omega;
@@ -281,11 +360,50 @@ int launch_vertex_field(cpic_run* r) {
     return CPIC_OK;
 }
 
-int launch_rhs(cpic_run* r, double* b) {
+namespace {
+
+FoldParams make_fold_params(const cpic_run* r) {
+    FoldParams f;
+    for (int a = 0; a < 3; ++a) {
+        f.n[a] = r->n[a];
+        const bool per = a < r->D && r->cfg.particle_bc[2 * a] == CPIC_PBC_PERIODIC;
+        f.lo[a] = per ? r->n[a] - 1 : 0;
+        f.hi[a] = per ? 0 : r->n[a] - 1;
+    }
+    f.hs1 = r->n[0] + 2;
+    f.hs2 = (r->n[0] + 2) * (r->n[1] + 2);
+    f.nsp = r->cfg.n_species;
+    f.ncell = r->ncell;
+    f.ncell_h = r->ncell_h;
+    f.src = r->charge_h;
+    f.dst = r->charge;
+    return f;
+}
+
+template <bool RHS>
+int launch_fold_kernel(cpic_run* r, double* b, const SolveReset& z) {
+    const FoldParams f = make_fold_params(r);
+    const RhsParams p = make_rhs_params(r);
+    const long long rows = (long long)r->n[1] * (r->D == 3 ? r->n[2] : 1);
+    long long nb = (rows + 7) / 8;
+    if (nb > 8LL * device_sm_count()) nb = 8LL * device_sm_count();
+    if (r->D == 2) fold_kernel<2, RHS><<<(int)nb, dim3(32, 8), 0, r->stream>>>(f, p, b, z);
+    else fold_kernel<3, RHS><<<(int)nb, dim3(32, 8), 0, r->stream>>>(f, p, b, z);
+    CPIC_CHECK_LAUNCH();
+    return CPIC_OK;
+}
+
+}  // namespace
+
+int launch_fold(cpic_run* r) { return launch_fold_kernel<false>(r, nullptr, SolveReset{}); }
+
+int launch_rhs(cpic_run* r, double* b, bool fold, int* done, unsigned* ticket) {
+    const SolveReset z{r->ctr, done, ticket};
+    if (fold) return launch_fold_kernel<true>(r, b, z);
     RhsParams p = make_rhs_params(r);
     long long nb = (r->ncell + 255) / 256;
     if (nb > 8LL * device_sm_count()) nb = 8LL * device_sm_count();
-    rhs_kernel<<<(int)nb, 256, 0, r->stream>>>(p, b);
+    rhs_kernel<<<(int)nb, 256, 0, r->stream>>>(p, b, z);
     CPIC_CHECK_LAUNCH();
     return CPIC_OK;
 }
@@ -311,10 +429,9 @@ int launch_floating_capacity(cpic_run* r) {
 
 int launch_field_energy(cpic_run* r) {
     RhsParams p = make_rhs_params(r);
-    const int nb = 256;
-    field_energy_partial<<<nb, 256, 0, r->stream>>>(p, r->lev[0].x, r->red);
-    CPIC_CHECK_LAUNCH();
-    field_energy_final<<<1, 32, 0, r->stream>>>(r->red, nb, r->ctr);
+    long long nb = (r->ncell + 255) / 256;
+    if (nb > ENERGY_BLOCKS) nb = ENERGY_BLOCKS;
+    field_energy_kernel<<<(int)nb, 256, 0, r->stream>>>(p, r->lev[0].x, r->red, r->ticket + 3, r->ctr);
     CPIC_CHECK_LAUNCH();
     return CPIC_OK;
 }

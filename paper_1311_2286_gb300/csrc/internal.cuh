@@ -253,7 +253,10 @@ int launch_map_analytic(cpic_run* r, int map_id, const double* params, int npara
 int launch_geometry(cpic_run* r);
 // fields.cu
 int launch_vertex_field(cpic_run* r);
-int launch_rhs(cpic_run* r, double* b);
+// charge -> right-hand side and the solve's counters reset; fold: from the padded deposit grid,
+// folding it into the compact one in the same pass
+int launch_rhs(cpic_run* r, double* b, bool fold, int* done, unsigned* ticket);
+int launch_fold(cpic_run* r);
 int launch_field_energy(cpic_run* r);
 // floating conductor: Gauss's-law potential of the face's conductor, then phi += V psi
 int launch_floating(cpic_run* r);
@@ -264,7 +267,6 @@ int launch_push(cpic_run* r);
 int launch_deposit(cpic_run* r);
 int launch_kick(cpic_run* r, double fraction);
 int launch_finalize_step(cpic_run* r);
-int launch_fold(cpic_run* r);
 int launch_push_prep(cpic_run* r);    // zero the deposit grid and kinetic-energy tallies
 int launch_push_kernel(cpic_run* r);  // the fused push + deposit kernel alone
 PushParams make_push_params(cpic_run* r);
@@ -278,14 +280,14 @@ int launch_push2d_batch(const PushParams* runs, const int* vbase, int nruns, int
 bool push2d_batchable(const cpic_run* r);
 // one step's work split around the particle push (for the batched launch): vertex field and
 // the zeroing of the deposit grid (and the push itself for runs that cannot join it); then
-// the step counter, injection, halo fold and sort
+// the step counter, injection and sort
 int enqueue_step_pre(cpic_run* r, bool with_push);
-int enqueue_step_post(cpic_run* r, bool sort, bool fold, bool fused_sort = false);
+int enqueue_step_post(cpic_run* r, bool sort, bool fused_sort = false);
 // a fused sort step: the push and the injection count the sort's histogram (zeroed here)
 int begin_counted_step(cpic_run* r);
 int launch_push3d(cpic_run* r, const PushParams& p);  // CPIC_ERR_NOT_BUILT: no specialisation
 // one PIC step without the field solve, enqueued on r->stream (also inside stream capture)
-int enqueue_step(cpic_run* r, bool sort, bool fold);
+int enqueue_step(cpic_run* r, bool sort);
 int count_kernel_nodes(cudaGraph_t g, int* out);
 int launch_load_maxwellian(cpic_run* r, int sp, long long n, double vth, const double* drift, unsigned long long seed);
 // inject.cu
@@ -301,10 +303,11 @@ bool push_fused_ok(const cpic_run* r);
 bool push3d_direct_taken(const cpic_run* r);
 // mg.cu
 int mg_setup(cpic_run* r);
-int mg_solve(cpic_run* r, double rtol, int max_cycles, bool host_loop, int* cycles, double* res);
+// fold: the charge is still in the padded deposit grid
+int mg_solve(cpic_run* r, double rtol, int max_cycles, bool fold, int* cycles, double* res);
 // enqueue the whole solve on the stream being captured into graph `g` after `deps`;
 // returns the node the rest of the step must depend on
-int mg_capture_solve(cpic_run* r, cudaGraph_t g, double rtol, int max_cycles);
+int mg_capture_solve(cpic_run* r, cudaGraph_t g, double rtol, int max_cycles);  // folds the charge
 void invalidate_graphs(cpic_run* r);
 // mg_cluster.cu
 int mg_cluster_prepare(cpic_run* r);

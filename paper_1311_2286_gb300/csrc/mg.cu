@@ -1366,7 +1366,7 @@ struct ResidualParams {
 
 // r = b - M phi in FP64, its FP32 copy, and ||r|| (and ||b|| with the first residual of a solve);
 // the last block to finish sums the block partials in a fixed order, updates the counters and
-// decides whether to continue. Blocks of 32 x 8 threads walk rows (j, k) of 32-cell segments.
+// decides whether to continue. A warp takes a row's segments of 32 cells.
 // Bound by the FP64 rate: 19 operations a cell for the 3D operator.
 template <int D, int NPT>
 __global__ void __launch_bounds__(256) residual_kernel(const __grid_constant__ ResidualParams P) {
@@ -1375,19 +1375,18 @@ __global__ void __launch_bounds__(256) residual_kernel(const __grid_constant__ R
     const LV<double>& L = P.L;
     const bool dot_rh = P.ks && !P.init, with_b = P.count_cycle == 0;
     double v[3] = {0.0, 0.0, 0.0};  // (r, r), (r^, r), (b, b)
-    const int nrows = L.n[1] * L.n[2];
-    for (int row = blockIdx.x * blockDim.y + threadIdx.y; row < nrows; row += gridDim.x * blockDim.y) {
-        int j = row % L.n[1], k = row / L.n[1];
-        for (int i = threadIdx.x; i < L.n[0]; i += blockDim.x) {
-            int q[3] = {i, j, k};
-            int c = i + L.n[0] * row;
-            const double b = L.b[c], r = b - stencil_sum<D, NPT, 0>(L, c, q);
-            if (P.r32) P.r32[c] = (float)r;
-            if (P.r64) P.r64[c] = r;
-            v[0] += r * r;
-            if (dot_rh) v[1] += P.rh[c] * r;
-            if (with_b) v[2] += b * b;
-        }
+    const int spr = (L.n[0] + 31) / 32, nseg = L.n[1] * L.n[2] * spr;
+    for (int w = blockIdx.x * blockDim.y + threadIdx.y; w < nseg; w += gridDim.x * blockDim.y) {
+        const int row = w / spr, i = (w - row * spr) * 32 + threadIdx.x;
+        if (i >= L.n[0]) continue;
+        const int k = row / L.n[1], q[3] = {i, row - k * L.n[1], k};
+        const int c = i + L.n[0] * row;
+        const double b = L.b[c], r = b - stencil_sum<D, NPT, 0>(L, c, q);
+        if (P.r32) P.r32[c] = (float)r;
+        if (P.r64) P.r64[c] = r;
+        v[0] += r * r;
+        if (dot_rh) v[1] += P.rh[c] * r;
+        if (with_b) v[2] += b * b;
     }
     block_sums<3>(v, sh);
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
@@ -1494,9 +1493,11 @@ __global__ void __launch_bounds__(256) bicg_matvec_kernel(const __grid_constant_
         // four consecutive cells along axis 0 per thread: each stencil entry of the four is one
         // 16-byte load, and a neighbour row's four values one 16-byte load plus the value
         // beyond the end the shifted entries need; the per-cell sums are stencil_apply's
-        const int n0 = L.n[0], q4 = n0 / 4;
-        for (int row = blockIdx.x * blockDim.y + threadIdx.y; row < nrows; row += gridDim.x * blockDim.y) {
-            const int j = row % L.n[1], k = row / L.n[1];
+        const int n0 = L.n[0], spr = (n0 + 127) / 128, nseg = nrows * spr;
+        for (int w = blockIdx.x * blockDim.y + threadIdx.y; w < nseg; w += gridDim.x * blockDim.y) {
+            const int row = w / spr, i0 = ((w - row * spr) * 32 + threadIdx.x) * 4;
+            if (i0 >= n0) continue;
+            const int k = row / L.n[1], j = row - k * L.n[1];
             int lo[3], hi[3];
             const int qq[3] = {0, j, k};
 #pragma unroll
@@ -1512,8 +1513,7 @@ __global__ void __launch_bounds__(256) bicg_matvec_kernel(const __grid_constant_
                 kz[1] = pl * k;
                 kz[2] = pl * hi[2];
             }
-            for (int g = threadIdx.x; g < q4; g += blockDim.x) {
-                const int i0 = 4 * g;
+            {
                 const int il = i0 > 0 ? i0 - 1 : (L.per[0] ? n0 - 1 : 0);
                 const int ir = i0 + 4 < n0 ? i0 + 4 : (L.per[0] ? 0 : n0 - 1);
                 const int c = i0 + n0 * row;
@@ -1641,15 +1641,6 @@ __global__ void gauge_kernel(LV<double> L, const double* part, int nb, double su
     if (threadIdx.x == 0) shift = s / sumJ;
     __syncthreads();
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < L.ncell; c += gridDim.x * blockDim.x) L.x[c] -= shift;
-}
-
-__global__ void reset_solve_kernel(DevCounters* ctr, int* done, unsigned* ticket) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        *done = 0;
-        *ticket = 0;
-        ctr->mg_cycles = 0;
-        ctr->mg_converged = 0;
-    }
 }
 
 // ------------------------------------------------------------------ setup kernels
@@ -1937,11 +1928,13 @@ size_t cta_smem_bytes(const LVSet& S, int* dense) {
 
 int* done_flag(cpic_run* r) { return reinterpret_cast<int*>(r->red + 3 * KRY_BLOCKS + 2); }
 
-// blocks of a pass over the finest level's rows of cells (kCellBlock: eight rows a block)
-int row_blocks(const cpic_run* r) {
+// blocks of a pass over the finest level in segments of rows, eight warps a block: one segment a
+// warp up to some three blocks an SM, four a warp beyond (each block ends with FP64 sums, 0.4 us)
+int row_blocks(const cpic_run* r, int segment) {
     const long long rows = (long long)r->lev[0].n[1] * (r->D == 3 ? r->lev[0].n[2] : 1);
-    const long long b = (rows + 7) / 8;
-    return (int)(b < 1 ? 1 : (b > KRY_BLOCKS ? KRY_BLOCKS : b));
+    const long long b = (rows * ((r->lev[0].n[0] + segment - 1) / segment) + 7) / 8;
+    const long long few = b < 512 ? b : (b / 4 > 512 ? b / 4 : 512);
+    return (int)(few > KRY_BLOCKS ? KRY_BLOCKS : few);
 }
 
 const dim3 kCellBlock(32, 8, 1);
@@ -2205,7 +2198,7 @@ int enqueue_residual(cpic_run* r, double rtol, int max_cycles, int count_cycle, 
     P.use_handle = use_handle ? 1 : 0;
     P.handle = h;
     return dispatch_shape(r, [&](auto Dc, auto Nc) -> int {
-        residual_kernel<decltype(Dc)::value, decltype(Nc)::value><<<row_blocks(r), kCellBlock, 0, r->stream>>>(P);
+        residual_kernel<decltype(Dc)::value, decltype(Nc)::value><<<row_blocks(r, 32), kCellBlock, 0, r->stream>>>(P);
         CPIC_CHECK_LAUNCH();
         return CPIC_OK;
     });
@@ -2231,7 +2224,7 @@ int enqueue_bicg_iteration(cpic_run* r, const LVSet& S, double rtol, int max_cyc
     LV<float> L0 = make_lv<float>(r, 0, true);  // A32 holds every entry of the operator
     e = dispatch_shape(r, [&](auto Dc, auto Nc) -> int {
         bicg_matvec_kernel<decltype(Dc)::value, decltype(Nc)::value>
-            <<<row_blocks(r), kCellBlock, 0, st>>>(L0, x32, 0, v, r->ph32, rh, nullptr, r->kry);
+            <<<row_blocks(r, r->n[0] % 4 ? 32 : 128), kCellBlock, 0, st>>>(L0, x32, 0, v, r->ph32, rh, nullptr, r->kry);
         CPIC_CHECK_LAUNCH();
         return CPIC_OK;
     });
@@ -2242,7 +2235,7 @@ int enqueue_bicg_iteration(cpic_run* r, const LVSet& S, double rtol, int max_cyc
     if (e) return e;
     e = dispatch_shape(r, [&](auto Dc, auto Nc) -> int {
         bicg_matvec_kernel<decltype(Dc)::value, decltype(Nc)::value>
-            <<<row_blocks(r), kCellBlock, 0, st>>>(L0, x32, 1, nullptr, nullptr, nullptr, s, r->kry);
+            <<<row_blocks(r, r->n[0] % 4 ? 32 : 128), kCellBlock, 0, st>>>(L0, x32, 1, nullptr, nullptr, nullptr, s, r->kry);
         CPIC_CHECK_LAUNCH();
         return CPIC_OK;
     });
@@ -2255,10 +2248,8 @@ int enqueue_bicg_iteration(cpic_run* r, const LVSet& S, double rtol, int max_cyc
 bool use_krylov(const cpic_run* r) { return r->solver == CPIC_SOLVER_BICGSTAB && !r->cluster_cs; }
 
 // right-hand side (and its projection); resets the solve counters
-int enqueue_prologue(cpic_run* r) {
-    reset_solve_kernel<<<1, 32, 0, r->stream>>>(r->ctr, done_flag(r), r->ticket);
-    CPIC_CHECK_LAUNCH();
-    int st = launch_rhs(r, r->lev[0].b);
+int enqueue_prologue(cpic_run* r, bool fold) {
+    int st = launch_rhs(r, r->lev[0].b, fold, done_flag(r), r->ticket);
     if (st) return st;
     if (r->singular) {
         LV<double> L0 = make_lv<double>(r, 0, false);
@@ -2380,10 +2371,9 @@ int mg_setup(cpic_run* r) {
 
 // Stream-ordered solve; the host reads the device decision after every cycle
 // (cpic_solve_field and the steps of an uncaptured cpic_step).
-int mg_solve(cpic_run* r, double rtol, int max_cycles, bool host_loop, int* cycles, double* res) {
-    (void)host_loop;
+int mg_solve(cpic_run* r, double rtol, int max_cycles, bool fold, int* cycles, double* res) {
     LVSet S = make_set(r);
-    int st = enqueue_prologue(r);
+    int st = enqueue_prologue(r, fold);
     if (st) return st;
     if (r->cluster_cs) {
         st = mg_cluster_solve(r, rtol, max_cycles);
@@ -2429,7 +2419,7 @@ int mg_solve(cpic_run* r, double rtol, int max_cycles, bool host_loop, int* cycl
 int mg_capture_solve(cpic_run* r, cudaGraph_t g, double rtol, int max_cycles) {
     LVSet S = make_set(r);
     if (r->cluster_cs) {
-        int st = enqueue_prologue(r);
+        int st = enqueue_prologue(r, true);
         if (st) return st;
         st = mg_cluster_solve(r, rtol, max_cycles);
         if (st) return st;
@@ -2437,7 +2427,7 @@ int mg_capture_solve(cpic_run* r, cudaGraph_t g, double rtol, int max_cycles) {
     }
     cudaGraphConditionalHandle h;
     CPIC_CUDA(cudaGraphConditionalHandleCreate(&h, g, 0, 0));
-    int st = enqueue_prologue(r);
+    int st = enqueue_prologue(r, true);
     if (st) return st;
     st = enqueue_residual(r, rtol, max_cycles, 0, true, h, use_krylov(r) ? 1 : 0);
     if (st) return st;

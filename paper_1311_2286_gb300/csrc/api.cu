@@ -221,6 +221,7 @@ void plan(cpic_run* r, Planner& P) {
     r->kv = P.take<double>((size_t)2 * r->ncell + ((size_t)3 * r->ncell + 1) / 2);  // r, r^; FP32 p, v, s
     r->ph32 = P.take<float>(r->ncell);
     r->hist = P.take<int>((size_t)c.n_species * r->ncell);
+    r->prank = P.take<int>(total);
     r->scan = P.take<long long>((size_t)c.n_species * r->ncell + 1);
     r->scan_blocks = P.take<long long>(1025);
     for (int l = 0; l < r->nlevels; ++l) {
@@ -615,8 +616,8 @@ int enqueue_step_post(cpic_run* r, bool sort, bool fused_sort) {
     return st;
 }
 
-// a fused sort step: the push and the injection count the particles' new cells, so the
-// sort skips its histogram pass
+// a fused sort step: the push and the injection count the particles' new cells and number the
+// particles of each, so the sort is a scan and a pass that looks their slots up
 int begin_counted_step(cpic_run* r) {
     r->count_hist = true;
     CPIC_CUDA(cudaMemsetAsync(r->hist, 0, sizeof(int) * r->cfg.n_species * (size_t)r->ncell, r->stream));

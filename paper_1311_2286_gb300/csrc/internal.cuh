@@ -121,7 +121,8 @@ struct PushParams {
     float gy[CPIC_MAX_SPECIES][4]; // per species cos th, sin th, sin th / th, (1 - cos th) / th
     int chunk;                     // particles per block chunk (0: one wave of blocks)
     int* hist;                     // when set: count each kept particle's new cell here
-                                   // ([species][cell], the next sort's histogram)
+                                   // ([species][cell], the next sort's histogram), and leave
+    int* rank;                     // the particle's number among its cell's per slot here
     int tile;                      // 1: shared-memory deposit tile when the chunk fits
     DevCounters* ctr;
 };
@@ -234,6 +235,7 @@ struct cpic_run {
     float* ph32;                 // preconditioned direction p_hat (FP32)
     // sort scratch
     int* hist;                   // [nsp][ncell] counts -> cursors
+    int* prank;                  // [slot] a particle's number among its cell's (counted steps)
     long long* scan;             // [nsp*ncell + 1] exclusive prefix
     long long* scan_blocks;      // block partials
     // injection

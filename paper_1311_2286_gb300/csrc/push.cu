@@ -423,6 +423,7 @@ PushParams make_push_params(cpic_run* r) {
     p.ctr = r->ctr;
     p.chunk = r->push_chunk;
     p.hist = r->count_hist ? r->hist : nullptr;
+    p.rank = r->prank;
     p.tile = r->push_tile;
     set_boris_constants(r, &p, 1.0);
     return p;

@@ -88,8 +88,9 @@ __device__ __forceinline__ void tile_add_row(unsigned& m, unsigned a, unsigned q
 // Deposit of one particle per lane into the chunk's tile; lanes whose 3x3 stencil leaves the
 // tile rows deposit straight into the padded global grid. Lanes that share a cell are summed
 // first (__reduce_add_sync over each such group) and deposited by one lane of the group.
+// peers: the lanes of this lane's new cell (alive lanes; the others hold keys of their own).
 __device__ __forceinline__ void deposit_tile(const PushParams& p, const Tile& tl, int s, bool alive,
-                                             const int* c, const float* t) {
+                                             const int* c, const float* t, unsigned peers) {
     const int lane = threadIdx.x & 31;
     const int rr = c[1] - tl.r0;  // tile row of the cell
     const bool in = alive && rr >= 1 && rr + 1 < tl.R;
@@ -98,10 +99,9 @@ __device__ __forceinline__ void deposit_tile(const PushParams& p, const Tile& tl
     if (!__any_sync(FULL, in)) return;
     unsigned q[9];
     node_weights<2>(t, q);
-    // lanes that do not deposit here get keys of their own; every group of lanes that share a
-    // cell is summed over its lanes and deposited by its lowest lane
-    const int off = in ? rr * tl.W + c[0] + 1 : -1 - lane;
-    const unsigned peers = __match_any_sync(FULL, off);
+    // every group of lanes that share a cell (all of them in the tile or none) is summed over its
+    // lanes and deposited by its lowest lane
+    const int off = rr * tl.W + c[0] + 1;
     const int my_leader = __ffs(peers) - 1;
     const bool issue = in && lane == my_leader;
     for (unsigned g = __ballot_sync(FULL, issue && (peers & (peers - 1u)) != 0u); g; g &= g - 1u) {
@@ -159,9 +159,13 @@ __device__ __forceinline__ void push2d_run(const PushParams& p, int bid, int nb,
         total += cnt[s];
     }
     if (total == 0) return;
-    // chunk size: a multiple of the block, about one chunk per block unless set
-    const int C = p.chunk > 0 ? p.chunk
-                              : ((total + nb - 1) / nb + P2_THREADS - 1) / P2_THREADS * P2_THREADS;
+    // chunk size: a multiple of the block. Unless set, a block's share is cut into equal chunks of at most AUTO_CHUNK particles: the blocks
+    // then work in a window that advances through the particles, and what a push reads through a
+    // pending order across chunks (a particle that moved a row) is still in L2 when its own
+    // chunk comes (64M particles on 512 x 1024: one chunk a block 1672 us, 8192: 1452 us, 1024: 1749)
+    constexpr int AUTO_CHUNK = 8192;
+    const int share = (total + nb - 1) / nb, cuts = (share + AUTO_CHUNK - 1) / AUTO_CHUNK;
+    const int C = p.chunk > 0 ? p.chunk : ((share + cuts - 1) / cuts + P2_THREADS - 1) / P2_THREADS * P2_THREADS;
     const int n0 = p.n[0], n1 = p.n[1], nv0 = n0 + 1;
     const float4* __restrict__ K4 = reinterpret_cast<const float4*>(p.K);
     const float2* __restrict__ G2 = reinterpret_cast<const float2*>(p.G);
@@ -380,19 +384,22 @@ __device__ __forceinline__ void push2d_run(const PushParams& p, int bid, int nb,
                 // spec D: v_old . v_new as an FP32 fma chain, then round(x 2^24) to int64
                 const float ke32 = __fmaf_rn(vo2, v[2], __fmaf_rn(vo1, v[1], __fmul_rn(vo0, v[0])));
                 if (active) ke += __float2ll_rn(__fmul_rn(ke32, 16777216.0f));
-                if (p.hist) {  // the next sort's histogram: one atomic per run of equal cells
-                    const int key = alive ? cn[0] + n0 * cn[1] : -1;
-                    const unsigned peers = __match_any_sync(FULL, key);
-                    if (key >= 0 && (__ffs(peers) - 1) == (int)(threadIdx.x & 31))
-                        atomicAdd(p.hist + (size_t)s * n0 * n1 + key, (int)__popc(peers));
-                }
+                const int lane = threadIdx.x & 31, key = alive ? cn[0] + n0 * cn[1] : -1 - lane;
+                const unsigned peers = __match_any_sync(FULL, key);
+                int number = 0;
+                if (p.hist && alive && __ffs(peers) - 1 == lane)  // the next sort's counts
+                    number = atomicAdd(p.hist + (size_t)s * n0 * n1 + key, (int)__popc(peers));
                 store_state(active, cellq + slot, alive ? (cn[0] | (cn[1] << 16)) : -1, tq + slot, tn[0],
                             tq + T + slot, tn[1], vq + slot, v[0], vq + T + slot, v[1], vq + 2 * T + slot, v[2]);
                 // a6: deposit
                 if constexpr (TILE)
-                    deposit_tile(p, tl, s, alive, cn, tn);
+                    deposit_tile(p, tl, s, alive, cn, tn, peers);
                 else
                     deposit_warp<2>(p, s, alive, cn, tn);
+                if (p.hist) {  // the particle's number among its cell's, once the atomic is back
+                    number = __shfl_sync(FULL, number, __ffs(peers) - 1);
+                    if (alive) p.rank[b0 + slot] = number + __popc(peers & ((1u << lane) - 1u));
+                }
             }
         };
         if (tl.on)

@@ -569,54 +569,102 @@ __global__ void __launch_bounds__(P3_THREADS, 3) push3d_kernel(PushParams p) {
 // ---------------------------------------------------------------- direct-deposit kernel
 // The same mover, with the b2 deposit going straight into the padded global grid through a
 // per-warp transposition: every lane writes its 27 node weights (spec Q) into its row of the
-// warp's shared buffer; then lane j (j < 27) walks the 32 rows, summing node j over each
-// run of consecutive lanes whose particles share a cell (particles are kept in cell order),
-// and adds the run's sum for node j with one 64-bit atomic when the run ends. A warp whose
-// 32 particles lie in one cell thus issues a single 27-lane atomic instruction; no lane
-// reduction instructions are needed, and the order of integer additions does not change
-// the result. No deposit tile: the kernel needs 28 KB of shared memory per block and runs
-// four blocks per SM.
+// warp's shared buffer; then lane j (j < 27) sums node j over the rows of each run of
+// consecutive lanes that came from one cell (particles are kept in cell order, so a warp has
+// one to three runs) and adds the run's sum with one 64-bit atomic. Particles that left
+// their cell are taken out of their run's sum and added at their own cell: runs of equal new
+// cells instead are cut by every such particle, twice (half the lanes' worth of 27-lane
+// atomics for electrons, a third of them move a cell per step). The order of integer additions
+// does not change the result. No deposit tile: the kernel needs 28 KB of shared memory per
+// block and runs four blocks per SM.
 constexpr int PD_THREADS = 256;
 constexpr int PD_STRIDE = 28;  // words per lane row: 27 node weights and one zero
 
+// old: padded offset of the cell the slot's particle came from (-1: empty slot); hist: the next
+// sort's counts of the species, or null; the particle's number among its new cell's goes to *rank
+// (the count's atomic returns it; it is stored last, so that its latency overlaps the deposit)
 __device__ __forceinline__ void deposit_runs3(const PushParams& p, int s, bool alive, const int* c, const float* t,
-                                              unsigned* wq) {
+                                              int old, unsigned* wq, int* hist, int* rank) {
     const int lane = threadIdx.x & 31;
     if (!__any_sync(FULL, alive)) return;
     unsigned w[3][3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) axis_weights(alive ? t[a] : 0.0f, w[a]);
+    for (int a = 0; a < 3; ++a) axis_weights(t[a], w[a]);
     // node weights in node order (m0 fastest), four to a 16-byte store; the centre (node 13)
-    // is written last, as 2^24 minus the other 26
+    // is written last, as 2^24 minus the other 26. The weight (w0 w12 + 2^23) >> 24 is the
+    // high word of (w0 2^8) w12 + 2^31; a lane without a particle has w0 = 0.
+#pragma unroll
+    for (int m = 0; m < 3; ++m) w[0][m] = alive ? w[0][m] << 8 : 0u;
     unsigned* row = wq + lane * PD_STRIDE;
     unsigned rest = 0, q4[4];
 #pragma unroll
     for (int node = 0; node < 28; ++node) {
         unsigned q = 0;
         if (node < 27 && node != 13) {
-            q = node_weight3(w[0][node % 3], w[1][(node / 3) % 3] * w[2][node / 9]);
+            const unsigned w12 = w[1][(node / 3) % 3] * w[2][node / 9];
+            q = (unsigned)(((unsigned long long)w[0][node % 3] * w12 + (1ull << 31)) >> 32);
             rest += q;
         }
-        q4[node & 3] = alive ? q : 0u;
+        q4[node & 3] = q;
         if ((node & 3) == 3) reinterpret_cast<uint4*>(row)[node >> 2] = make_uint4(q4[0], q4[1], q4[2], q4[3]);
     }
-    row[13] = alive ? (1u << QF) - rest : 0u;
+    row[13] = (alive ? 1u << QF : 0u) - rest;
     const int off = alive ? c[0] + c[1] * p.hs1 + c[2] * p.hs2 : -1;
-    const int next = __shfl_down_sync(FULL, off, 1);  // every lane takes part (lane 31 gets its own)
-    const unsigned ends = __ballot_sync(FULL, lane == 31 || next != off);
+    const int next = __shfl_down_sync(FULL, old, 1);  // every lane takes part (lane 31 gets its own)
+    unsigned ends = __ballot_sync(FULL, lane == 31 || next != old);
+    const unsigned stay = __ballot_sync(FULL, alive && off == old);
+    const unsigned move = __ballot_sync(FULL, alive && off != old);
+    int number = 0, first = lane;  // the atomic's value, held by lane `first`
+    unsigned mine = 0;
+    const bool mover = (move >> lane) & 1u;
+    if (hist) {
+        // the first of a run's stayers counts them all, a mover counts itself
+        const unsigned below = (1u << lane) - 1u, before = ends & below;
+        const int start = before ? 32 - __clz(before) : 0;
+        const int end = __ffs(ends & ~below) - 1;
+        mine = stay & ((2u << end) - 1u) & ~((1u << start) - 1u);
+        if (!mover && mine) first = __ffs(mine) - 1;
+        if (alive && first == lane)
+            number = atomicAdd(hist + c[0] + p.n[0] * (c[1] + p.n[1] * c[2]), mover ? 1 : __popc(mine));
+    }
     __syncwarp();
     const int j = lane < 27 ? lane : 27;  // lanes 27-31 read the zero word
     const int dj = (j % 3 - 1) + ((j / 3) % 3 - 1) * p.hs1 + (j / 9 - 1) * p.hs2;
     unsigned long long* g = p.charge + (long long)s * p.ncell_h + p.origin + dj;
-    unsigned acc = 0;
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        acc += wq[r * PD_STRIDE + j];
-        if ((ends >> r) & 1u) {  // warp-uniform
+    const unsigned* col = wq + j;
+    // the run of rows [a, e]: acc over all of them, less the movers, which go to their own cells
+    auto finish = [&](unsigned acc, unsigned rows, int e) {
+        for (unsigned m = move & rows; m; m &= m - 1u) {
+            const int r = __ffs(m) - 1;
+            const unsigned x = col[r * PD_STRIDE];
+            acc -= x;
             const int o = __shfl_sync(FULL, off, r);
-            if (o >= 0 && lane < 27) atomicAdd(g + o, (unsigned long long)acc);
-            acc = 0;
+            if (lane < 27) atomicAdd(g + o, (unsigned long long)x);
         }
+        if (stay & rows) {
+            const int o = __shfl_sync(FULL, old, e);
+            if (lane < 27) atomicAdd(g + o, (unsigned long long)acc);
+        }
+    };
+    if (ends == 0x80000000u) {
+        unsigned acc[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int r = 0; r < 32; ++r) acc[r & 3] += col[r * PD_STRIDE];
+        finish((acc[0] + acc[1]) + (acc[2] + acc[3]), FULL, 31);
+    } else {
+        int a = 0;
+        for (; ends; ends &= ends - 1u) {
+            const int e = __ffs(ends) - 1;
+            unsigned acc = 0;
+#pragma unroll 4
+            for (int r = a; r <= e; ++r) acc += col[r * PD_STRIDE];
+            finish(acc, ((2u << e) - 1u) & ~((1u << a) - 1u), e);
+            a = e + 1;
+        }
+    }
+    if (hist) {
+        number = __shfl_sync(FULL, number, first);
+        if (alive) *rank = mover ? number : number + __popc(mine & ((1u << lane) - 1u));
     }
     __syncwarp();  // the rows are read before the next particle's weights overwrite them
 }
@@ -672,16 +720,22 @@ __global__ void __launch_bounds__(PD_THREADS, 4) push3d_direct_kernel(PushParams
 
         long long ke = 0;
         int i = lo + (int)threadIdx.x;
+        int* hist = p.hist ? p.hist + (size_t)s * p.n[0] * p.n[1] * p.n[2] : nullptr;
         int ncw = -1;
         float nt[3] = {0.f, 0.f, 0.f}, nv[3] = {0.f, 0.f, 0.f};
-        if (i < hi) {
-            const int src = perm ? cellq[i] : i;
+        // the source index is loaded two iterations ahead and the state one, so that neither load
+        // waits for the other
+        auto index = [&](int k) { return perm && k < hi ? cellq[k] : k; };
+        auto fetch = [&](int src) {
             ncw = cellp[src];
 #pragma unroll
             for (int a = 0; a < 3; ++a) nt[a] = tq0[a * T + src];
 #pragma unroll
             for (int a = 0; a < 3; ++a) nv[a] = vq0[a * T + src];
-        }
+        };
+        int src = index(i);
+        if (i < hi) fetch(src);
+        src = index(i + PD_THREADS);
         for (int base = lo; base < hi; base += PD_THREADS) {
             const int slot = i;
             const int cw = ncw;
@@ -689,14 +743,8 @@ __global__ void __launch_bounds__(PD_THREADS, 4) push3d_direct_kernel(PushParams
             float v[3] = {nv[0], nv[1], nv[2]};
             i += PD_THREADS;
             ncw = -1;
-            if (i < hi) {
-                const int src = perm ? cellq[i] : i;
-                ncw = cellp[src];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) nt[a] = tq0[a * T + src];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) nv[a] = vq0[a * T + src];
-            }
+            if (i < hi) fetch(src);
+            src = index(i + PD_THREADS);
             int cn[3], face;
             float tn[3], ke32;
             const bool active = cw >= 0;
@@ -707,15 +755,10 @@ __global__ void __launch_bounds__(PD_THREADS, 4) push3d_direct_kernel(PushParams
                 atomicAdd(&sh_gone[face], 1);
                 collect_face<3>(p, s, face, cn);
             }
-            if (p.hist) {  // the next sort's histogram: one atomic per run of equal cells
-                const int key = alive ? cn[0] + p.n[0] * (cn[1] + p.n[1] * cn[2]) : -1;
-                const unsigned peers = __match_any_sync(FULL, key);
-                if (key >= 0 && (__ffs(peers) - 1) == (int)(threadIdx.x & 31))
-                    atomicAdd(p.hist + (size_t)s * p.n[0] * p.n[1] * p.n[2] + key, (int)__popc(peers));
-            }
             store_state3(active, cellq + slot, alive ? (cn[0] | (cn[1] << 10) | (cn[2] << 20)) : -1, tq1 + slot,
                          tq1 + T + slot, tq1 + 2 * T + slot, tn, vq1 + slot, vq1 + T + slot, vq1 + 2 * T + slot, v);
-            deposit_runs3(p, s, alive, cn, tn, wq);  // a6
+            const int old = active ? (cw & 1023) + ((cw >> 10) & 1023) * p.hs1 + (cw >> 20) * p.hs2 : -1;
+            deposit_runs3(p, s, alive, cn, tn, old, wq, hist, p.rank + b0 + slot);  // a6
         }
         ke = warp_sum_ll(ke);
         if ((threadIdx.x & 31) == 0 && ke) atomicAdd((unsigned long long*)&p.ctr->ke_fp[s], (unsigned long long)ke);

@@ -371,6 +371,57 @@ __global__ void __launch_bounds__(256) gather_kernel(SortParams p) {
     p.ctr->perm = 0;
 }
 
+// After a counted step (the push and the injection have numbered the particles of each cell): a
+// particle's slot is its cell's start plus its number. The slot receives the particle's
+// source index, as in the rank pass; the last block to finish makes the live counts the sorted
+// ones and leaves the order pending (see launch_sort). Four particles a thread with 16-byte
+// loads. 64M particles on 128^3 cells: 170 us, against 537 us for the rank pass, which counts
+// every chunk's cells again (255 against 372 us on 512 x 1024, sorted every other step); the returned counts cost the push 5 %.
+template <int D>
+__global__ void __launch_bounds__(256) place_kernel(SortParams p, const int* __restrict__ rank) {
+    __shared__ bool last;
+    const int s = blockIdx.y, cur = p.ctr->cur;
+    const unsigned n = (unsigned)p.ctr->count[s];  // the loop steps past it: below 2^31 + 2^21
+    const long long b0 = p.pb.base[s];
+    const int* __restrict__ cin = p.pb.cell[cur] + b0;
+    const int* __restrict__ num = rank + b0;
+    int* __restrict__ cout = p.pb.cell[1 - cur] + b0;
+    const long long* __restrict__ scan = p.scan + (long long)s * p.ncell;
+    const long long first = scan[0];
+    const int n0 = p.n[0], n1 = p.n[1];
+    auto put = [&](int cw, int r, int i) {
+        if (cw < 0) return;
+        const int key = D == 2 ? (cw & 0xFFFF) + n0 * (cw >> 16) : (cw & 1023) + n0 * (((cw >> 10) & 1023) + n1 * (cw >> 20));
+        cout[(int)(__ldg(scan + key) - first) + r] = i;
+    };
+    for (unsigned i = 4u * (blockIdx.x * 256u + threadIdx.x); i < n; i += 4u * 256u * gridDim.x) {
+        if (i + 4 <= n) {
+            const int4 c = *reinterpret_cast<const int4*>(cin + i), r = *reinterpret_cast<const int4*>(num + i);
+            put(c.x, r.x, (int)i);
+            put(c.y, r.y, (int)i + 1);
+            put(c.z, r.z, (int)i + 2);
+            put(c.w, r.w, (int)i + 3);
+        } else {
+            for (unsigned k = i; k < n; ++k) put(cin[k], num[k], (int)k);
+        }
+    }
+    __syncthreads();  // every thread of the block has read the counters
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(p.ticket, 1u) == gridDim.x * gridDim.y - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x != 0) return;
+    __threadfence();
+    *p.ticket = 0;
+    for (int sp = 0; sp < p.nsp; ++sp) {
+        const long long cnt = p.scan[(long long)(sp + 1) * p.ncell] - p.scan[(long long)sp * p.ncell];
+        p.ctr->count[sp] = cnt;
+        p.ctr->alive[sp] = cnt;
+    }
+    p.ctr->perm = 1;
+}
+
 // Fused sort: the live counts become the sorted ones and the order is left pending; the next
 // push reads slot i's particle from the index the rank pass stored in the other buffer, writes
 // it to slot i there, and the step's finalisation flips the buffers.
@@ -431,9 +482,9 @@ int launch_sort(cpic_run* r, bool fused) {
     long long pblocks = (tot + 255) / 256;
     if (pblocks > 8LL * device_sm_count()) pblocks = 8LL * device_sm_count();
     if (pblocks < 1) pblocks = 1;
-    if (r->count_hist) {
-        r->count_hist = false;  // the step's push and injection counted the cells
-    } else {
+    const bool counted = r->count_hist;  // the step's push and injection counted the cells
+    r->count_hist = false;
+    if (!counted) {
         CPIC_CUDA(cudaMemsetAsync(r->hist, 0, sizeof(int) * N, r->stream));
         hist_kernel<<<(int)pblocks, 256, 0, r->stream>>>(p);
         CPIC_CHECK_LAUNCH();
@@ -447,6 +498,18 @@ int launch_sort(cpic_run* r, bool fused) {
     CPIC_CHECK_LAUNCH();
     scan_final_kernel<<<nb, SCAN_THREADS, 0, r->stream>>>(r->hist, N, chunk, r->scan_blocks, r->scan);
     CPIC_CHECK_LAUNCH();
+    if (counted && fused) {
+        long long most = 0;
+        for (int s = 0; s < p.nsp; ++s) most = r->pb.capacity[s] > most ? r->pb.capacity[s] : most;
+        long long nb = (most + 1023) / 1024, cap = 8LL * device_sm_count() / p.nsp;
+        nb = nb > cap ? cap : nb;
+        const dim3 grid((unsigned)(nb < 1 ? 1 : nb), (unsigned)p.nsp);
+        if (p.D == 2) place_kernel<2><<<grid, 256, 0, r->stream>>>(p, r->prank);
+        else place_kernel<3><<<grid, 256, 0, r->stream>>>(p, r->prank);
+        CPIC_CHECK_LAUNCH();
+        r->order_pending = true;
+        return CPIC_OK;
+    }
     CPIC_CUDA(cudaMemsetAsync(r->hist, 0, sizeof(int) * N, r->stream));
     if (p.D == 2)
         rank_kernel<2><<<(int)pblocks, 256, 0, r->stream>>>(p);

@@ -603,40 +603,26 @@ bool push2d_batchable(const cpic_run* r) {
 }
 
 int enqueue_step_pre(cpic_run* r, bool with_push) {
-    int st = launch_vertex_field(r);
-    if (!st) st = launch_push_prep(r);
+    int st = launch_vertex_field(r, true);
     if (!st && with_push) st = launch_push_kernel(r);
     return st;
 }
 
-int enqueue_step_post(cpic_run* r, bool sort, bool fused_sort) {
-    int st = launch_finalize_step(r);
+int enqueue_step_post(cpic_run* r, bool sort, bool finalized, bool fused_sort) {
+    int st = finalized ? CPIC_OK : launch_finalize_step(r);
     if (!st) st = launch_inject(r);
     if (!st && sort) st = launch_sort(r, fused_sort);
     return st;
 }
 
-// a fused sort step: the push and the injection count the particles' new cells and number the
-// particles of each, so the sort is a scan and a pass that looks their slots up
-int begin_counted_step(cpic_run* r) {
-    r->count_hist = true;
-    CPIC_CUDA(cudaMemsetAsync(r->hist, 0, sizeof(int) * r->cfg.n_species * (size_t)r->ncell, r->stream));
-    return CPIC_OK;
-}
-
+// one step without the solve. A fused sort step is a counted one: the push and the injection count
+// the particles' new cells and number the particles of each, so the sort is a scan and a pass
+// that looks their slots up.
 int enqueue_step(cpic_run* r, bool sort, bool fused_sort = false) {
-    int st = launch_vertex_field(r);
-    if (st) return st;
-    if (sort && fused_sort && (st = begin_counted_step(r))) return st;
-    st = launch_push(r);
-    if (st) return st;
-    st = launch_inject(r);
-    if (st) return st;
-    if (sort) {
-        st = launch_sort(r, fused_sort);
-        if (st) return st;
-    }
-    return CPIC_OK;
+    r->count_hist = sort && fused_sort;
+    int st = enqueue_step_pre(r, true);
+    if (!st) st = enqueue_step_post(r, sort, push_finalizes(r), fused_sort);
+    return st;
 }
 
 namespace {
@@ -738,16 +724,13 @@ int step_once(cpic_run* r, bool solve) {
     // profiled path: the same work launched stream-ordered, bracketed by events; the push
     // phase holds the fused push kernel alone
     const bool fused = sort && push_fused_ok(r);
-    int st = phase(r, CPIC_PHASE_FIELD, [&] {
-        int q = launch_vertex_field(r);
-        if (!q && fused) q = begin_counted_step(r);
-        return q ? q : launch_push_prep(r);
-    });
+    r->count_hist = fused;
+    int st = phase(r, CPIC_PHASE_FIELD, [&] { return launch_vertex_field(r, true); });
     if (st) return st;
     st = phase(r, CPIC_PHASE_PUSH, [&] { return launch_push_kernel(r); });
     if (st) return st;
     st = phase(r, CPIC_PHASE_INJECT, [&] {
-        const int q = launch_finalize_step(r);
+        const int q = push_finalizes(r) ? CPIC_OK : launch_finalize_step(r);
         return q ? q : launch_inject(r);
     });
     if (st) return st;

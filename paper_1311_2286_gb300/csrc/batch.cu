@@ -138,8 +138,8 @@ int capture(cpic_batch* b, bool solve, const std::string& key, cpic_batch::Graph
         }
         cudaStream_t saved = r->stream;
         r->stream = b->branch[i];
-        if (out->fused[i]) st = begin_counted_step(r);
-        if (!st) st = enqueue_step_pre(r, !persistent || !push2d_batchable(r));
+        r->count_hist = out->fused[i] != 0;
+        st = enqueue_step_pre(r, !persistent || !push2d_batchable(r));
         r->stream = saved;
         if (st) break;
         e = cudaEventRecord(b->join_pre[i], b->branch[i]);
@@ -168,7 +168,7 @@ int capture(cpic_batch* b, bool solve, const std::string& key, cpic_batch::Graph
         }
         cudaStream_t saved = r->stream;
         r->stream = b->branch[i];
-        st = enqueue_step_post(r, key[i] == '1', out->fused[i] != 0);
+        st = enqueue_step_post(r, key[i] == '1', !(persistent && push2d_batchable(r)) && push_finalizes(r), out->fused[i] != 0);
         if (!st && solve) {
             cudaStreamCaptureStatus cs;
             cudaGraph_t cg = nullptr;

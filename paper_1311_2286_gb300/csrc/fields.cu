@@ -48,18 +48,34 @@ __device__ __forceinline__ double phi_ext(const FieldGrid& g, const double* __re
     return val;
 }
 
+// What the next push accumulates into, zeroed in the same pass (memset nodes cost a microsecond and
+// a half each, and their writes overlap this kernel's FP64 work)
+struct ZeroParams {
+    uint4* charge;
+    int* hist;         // null: this step does not count
+    long long ncharge, nhist;  // 16-byte words, words
+    unsigned long long* charge_tail;  // the last count when their number is odd, else null
+    long long* ke;     // null: nothing to zero
+};
+
 // 3D: G is also written into the three padding words of each vertex's k record (K[12 v + 9 ..
 // 11]), so that the mover's first gather reads k and G in three 16-byte loads per corner.
-__global__ void vertex_field_kernel(FieldGrid g, const double* __restrict__ phi, float* G, float* K) {
+__global__ void __launch_bounds__(256) vertex_field_kernel(FieldGrid g, const double* __restrict__ phi, float* G, float* K,
+                                                           const __grid_constant__ ZeroParams z) {
     if (g.fface >= 0) g.bcv[g.fface] = *g.fphi;
-    long long nv0 = g.n[0] + 1, nv1 = g.n[1] + 1, nv2 = g.D == 3 ? g.n[2] + 1 : 1;
-    long long nvt = nv0 * nv1 * nv2;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nvt;
-         v += (long long)gridDim.x * blockDim.x) {
-        int i = (int)(v % nv0);
-        long long rest = v / nv0;
-        int j = (int)(rest % nv1);
-        int k = (int)(rest / nv1);
+    const unsigned first = blockIdx.x * 256u + threadIdx.x, step = gridDim.x * 256u;
+    if (z.ke) {
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        for (long long e = first; e < z.ncharge; e += step) z.charge[e] = zero;
+        if (z.hist)
+            for (long long e = first; e < z.nhist; e += step) z.hist[e] = 0;
+        if (first < CPIC_MAX_SPECIES) z.ke[first] = 0;
+        if (first == 0 && z.charge_tail) *z.charge_tail = 0;
+    }
+    const unsigned nv0 = g.n[0] + 1, nv1 = g.n[1] + 1, nvt = nv0 * nv1 * (g.D == 3 ? g.n[2] + 1 : 1);
+    for (unsigned v = first; v < nvt; v += step) {
+        const unsigned rest = v / nv0;
+        const int i = (int)(v - rest * nv0), k = g.D == 3 ? (int)(rest / nv1) : 0, j = (int)(rest - k * nv1);
         if (g.D == 2) {
             double p00 = phi_ext(g, phi, i - 1, j - 1, 0);
             double p01 = phi_ext(g, phi, i, j - 1, 0);
@@ -88,7 +104,7 @@ __global__ void vertex_field_kernel(FieldGrid g, const double* __restrict__ phi,
                 out[a] = __double2float_rn(__dmul_rn(acc, 0.25));
             }
             reinterpret_cast<float4*>(G)[v] = make_float4(out[0], out[1], out[2], 0.0f);
-            float* kr = K + 12 * v;
+            float* kr = K + 12ull * v;
             kr[9] = out[0];
             kr[10] = out[1];
             kr[11] = out[2];
@@ -351,11 +367,21 @@ RhsParams make_rhs_params(const cpic_run* r) {
     return p;
 }
 
-int launch_vertex_field(cpic_run* r) {
+int launch_vertex_field(cpic_run* r, bool prep) {
     FieldGrid g = make_field_grid(r);
+    ZeroParams z = {};
+    if (prep) {
+        const long long n = r->ncell_h * r->cfg.n_species;
+        z.charge = reinterpret_cast<uint4*>(r->charge_h);
+        z.ncharge = n / 2;
+        z.charge_tail = n & 1 ? r->charge_h + n - 1 : nullptr;
+        z.hist = r->count_hist ? r->hist : nullptr;
+        z.nhist = r->ncell * r->cfg.n_species;
+        z.ke = r->ctr->ke_fp;
+    }
     long long b = (r->nvert + 255) / 256;
     if (b > 8LL * device_sm_count()) b = 8LL * device_sm_count();
-    vertex_field_kernel<<<(int)b, 256, 0, r->stream>>>(g, r->lev[0].x, r->G32, r->K32);
+    vertex_field_kernel<<<(int)b, 256, 0, r->stream>>>(g, r->lev[0].x, r->G32, r->K32, z);
     CPIC_CHECK_LAUNCH();
     return CPIC_OK;
 }

@@ -124,6 +124,8 @@ struct PushParams {
                                    // ([species][cell], the next sort's histogram), and leave
     int* rank;                     // the particle's number among its cell's per slot here
     int tile;                      // 1: shared-memory deposit tile when the chunk fits
+    unsigned* fin;                 // when set: block counter, the last block to finish ends the
+                                   // step's push (step count, buffer flip of a pending order)
     DevCounters* ctr;
 };
 
@@ -254,7 +256,9 @@ namespace cpic {
 int launch_map_analytic(cpic_run* r, int map_id, const double* params, int nparams);
 int launch_geometry(cpic_run* r);
 // fields.cu
-int launch_vertex_field(cpic_run* r);
+// prep: also zero what the push accumulates into (deposit grid, kinetic energy, and the sort's
+// counts on a counted step)
+int launch_vertex_field(cpic_run* r, bool prep = false);
 // charge -> right-hand side and the solve's counters reset; fold: from the padded deposit grid,
 // folding it into the compact one in the same pass
 int launch_rhs(cpic_run* r, double* b, bool fold, int* done, unsigned* ticket);
@@ -271,6 +275,8 @@ int launch_kick(cpic_run* r, double fraction);
 int launch_finalize_step(cpic_run* r);
 int launch_push_prep(cpic_run* r);    // zero the deposit grid and kinetic-energy tallies
 int launch_push_kernel(cpic_run* r);  // the fused push + deposit kernel alone
+// whether that kernel also ends the push (else launch_finalize_step follows it)
+bool push_finalizes(const cpic_run* r);
 PushParams make_push_params(cpic_run* r);
 void set_boris_constants(const cpic_run* r, PushParams* p, double fraction);
 int launch_push2d(cpic_run* r, const PushParams& p);
@@ -284,9 +290,7 @@ bool push2d_batchable(const cpic_run* r);
 // the zeroing of the deposit grid (and the push itself for runs that cannot join it); then
 // the step counter, injection and sort
 int enqueue_step_pre(cpic_run* r, bool with_push);
-int enqueue_step_post(cpic_run* r, bool sort, bool fused_sort = false);
-// a fused sort step: the push and the injection count the sort's histogram (zeroed here)
-int begin_counted_step(cpic_run* r);
+int enqueue_step_post(cpic_run* r, bool sort, bool finalized, bool fused_sort = false);
 int launch_push3d(cpic_run* r, const PushParams& p);  // CPIC_ERR_NOT_BUILT: no specialisation
 // one PIC step without the field solve, enqueued on r->stream (also inside stream capture)
 int enqueue_step(cpic_run* r, bool sort);

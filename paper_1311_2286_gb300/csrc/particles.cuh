@@ -299,6 +299,28 @@ __device__ __forceinline__ int species_of(const SpeciesRanges& r, int vi, long l
     return s;
 }
 
+// End of a push: the step count, and the buffer flip of a push that read through a pending sort
+// order and wrote the other buffer
+__device__ __forceinline__ void end_push(DevCounters* ctr) {
+    ctr->step += 1;
+    if (ctr->perm) {
+        ctr->cur = 1 - ctr->cur;
+        ctr->perm = 0;
+    }
+}
+// by the last block of the kernel to get here (a launch of its own costs two microseconds a step).
+// Every thread of the block calls it, after its last use of the counters. No fence: the last
+// block only overwrites what the others have read (a fence here waits for every block's state
+// stores and deposits to settle, 200 us of a 1500 us push).
+__device__ __forceinline__ void end_push_last_block(const PushParams& p) {
+    if (!p.fin) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    if (atomicAdd(p.fin, 1u) != gridDim.x - 1) return;
+    *p.fin = 0u;
+    end_push(p.ctr);
+}
+
 __device__ __forceinline__ long long warp_sum_ll(long long v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);

@@ -386,15 +386,9 @@ __global__ void __launch_bounds__(256, D == 2 ? 4 : 2) particle_kernel(PushParam
     if (MODE == 0 && s_acc >= 0) tally.flush(p.ctr, s_acc);
 }
 
-// step count; a push that read through a pending sort order wrote the other buffer: flip
+// the end of a push whose kernel does not see to it (the generic one, the batched one)
 __global__ void finalize_step_kernel(DevCounters* ctr) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        ctr->step += 1;
-        if (ctr->perm) {
-            ctr->cur = 1 - ctr->cur;
-            ctr->perm = 0;
-        }
-    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) end_push(ctr);
 }
 
 }  // namespace
@@ -425,6 +419,7 @@ PushParams make_push_params(cpic_run* r) {
     p.hist = r->count_hist ? r->hist : nullptr;
     p.rank = r->prank;
     p.tile = r->push_tile;
+    p.fin = nullptr;
     set_boris_constants(r, &p, 1.0);
     return p;
 }
@@ -528,6 +523,17 @@ bool push_fused_ok(const cpic_run* r) {
     return true;
 }
 
+bool push_finalizes(const cpic_run* r) {
+    if (r->magnetized) return false;
+    if (r->D == 3) {
+        const int k0 = r->cfg.particle_bc[0], k1 = r->cfg.particle_bc[2], k2 = r->cfg.particle_bc[4];
+        return (k0 == CPIC_PBC_ABSORB && k1 == CPIC_PBC_REFLECT && k2 == CPIC_PBC_PERIODIC) ||
+               (k0 == CPIC_PBC_PERIODIC && k1 == CPIC_PBC_PERIODIC && k2 == CPIC_PBC_PERIODIC);
+    }
+    return !r->cfg.axisymmetric && r->cfg.particle_bc[0] != CPIC_PBC_REFLECT && r->cfg.particle_bc[1] != CPIC_PBC_REFLECT &&
+           r->cfg.particle_bc[2] != CPIC_PBC_REFLECT && r->cfg.particle_bc[3] != CPIC_PBC_REFLECT;
+}
+
 int launch_push_kernel(cpic_run* r) {
     // a pending sort order: the direct 3D kernel and the 2D kernel read through it (the step's
     // finalisation flips the buffers); any other kernel needs the particles gathered first
@@ -544,9 +550,11 @@ int launch_push_kernel(cpic_run* r) {
     for (int f = 0; f < 2 * r->D; ++f) reflect = reflect || r->cfg.particle_bc[f] == CPIC_PBC_REFLECT;
     // Boris kick and the axisymmetric mover: the generic kernel
     if (r->magnetized || (r->D == 2 && r->cfg.axisymmetric)) return launch_particles<0>(r, 0, 0, 0, 0);
-    if (r->D == 2 && !reflect) return launch_push2d(r, make_push_params(r));
+    PushParams p = make_push_params(r);
+    p.fin = r->ticket + 1;
+    if (r->D == 2 && !reflect) return launch_push2d(r, p);
     if (r->D == 3) {
-        const int st = launch_push3d(r, make_push_params(r));
+        const int st = launch_push3d(r, p);
         if (st != CPIC_ERR_NOT_BUILT) return st;
     }
     return launch_particles<0>(r, 0, 0, 0, 0);
@@ -555,7 +563,7 @@ int launch_push_kernel(cpic_run* r) {
 int launch_push(cpic_run* r) {
     int st = launch_push_prep(r);
     if (!st) st = launch_push_kernel(r);
-    if (st) return st;
+    if (st || push_finalizes(r)) return st;
     return launch_finalize_step(r);
 }
 

@@ -448,6 +448,7 @@ __global__ void __launch_bounds__(P2_THREADS, 4) push2d_kernel(PushParams p) {
     __shared__ unsigned tile_lo[TILE_CELLS], tile_hi[TILE_CELLS];
     __shared__ int red_min[P2_THREADS / 32], red_max[P2_THREADS / 32];
     push2d_run<PER0, PER1>(p, (int)blockIdx.x, (int)gridDim.x, tile_lo, tile_hi, red_min, red_max);
+    end_push_last_block(p);
 }
 
 // Row a11: the particle step of many runs in one persistent launch. Run r owns virtual

@@ -345,7 +345,10 @@ __global__ void __launch_bounds__(P3_THREADS, 3) push3d_kernel(PushParams p) {
         cnt[s] = s < nsp ? (int)ctr->count[s] : 0;
         total += cnt[s];
     }
-    if (total == 0) return;
+    if (total == 0) {
+        end_push_last_block(p);
+        return;
+    }
     int C = ((total + (int)gridDim.x - 1) / (int)gridDim.x + P3_THREADS - 1) / P3_THREADS * P3_THREADS;
     if (C > P3_CHUNK) C = P3_CHUNK;
     if (p.chunk > 0) C = p.chunk;
@@ -564,6 +567,7 @@ __global__ void __launch_bounds__(P3_THREADS, 3) push3d_kernel(PushParams p) {
             if (removed) atomicAdd((unsigned long long*)&cw->alive[s], (unsigned long long)(-removed));
         }
     }
+    end_push_last_block(p);
 }
 
 // ---------------------------------------------------------------- direct-deposit kernel
@@ -576,7 +580,10 @@ __global__ void __launch_bounds__(P3_THREADS, 3) push3d_kernel(PushParams p) {
 // cells instead are cut by every such particle, twice (half the lanes' worth of 27-lane
 // atomics for electrons, a third of them move a cell per step). The order of integer additions
 // does not change the result. No deposit tile: the kernel needs 28 KB of shared memory per
-// block and runs four blocks per SM.
+// block. Three blocks per SM at 80 registers: at 64 it spills (64M particles with the sort's
+// numbers: 3084 us against 3196 with four blocks). What is left is latency and the L1 data
+// pipe: without the second gather 490 us less, without the atomics 350, without the row sums
+// and movers 1160.
 constexpr int PD_THREADS = 256;
 constexpr int PD_STRIDE = 28;  // words per lane row: 27 node weights and one zero
 
@@ -670,7 +677,7 @@ __device__ __forceinline__ void deposit_runs3(const PushParams& p, int s, bool a
 }
 
 template <int K0, int K1, int K2>
-__global__ void __launch_bounds__(PD_THREADS, 4) push3d_direct_kernel(PushParams p) {
+__global__ void __launch_bounds__(PD_THREADS, 3) push3d_direct_kernel(PushParams p) {
     __shared__ __align__(16) unsigned qbuf[PD_THREADS / 32][32 * PD_STRIDE];
     __shared__ int sh_gone[8];  // removed particles of the chunk per face (6: non-finite)
     const DevCounters* ctr = p.ctr;
@@ -688,7 +695,10 @@ __global__ void __launch_bounds__(PD_THREADS, 4) push3d_direct_kernel(PushParams
         cnt[s] = s < nsp ? (int)ctr->count[s] : 0;
         total += cnt[s];
     }
-    if (total == 0) return;
+    if (total == 0) {
+        end_push_last_block(p);
+        return;
+    }
     int C = ((total + (int)gridDim.x - 1) / (int)gridDim.x + PD_THREADS - 1) / PD_THREADS * PD_THREADS;
     if (C > P3_CHUNK) C = P3_CHUNK;
     if (p.chunk > 0) C = p.chunk;
@@ -778,6 +788,7 @@ __global__ void __launch_bounds__(PD_THREADS, 4) push3d_direct_kernel(PushParams
             if (removed) atomicAdd((unsigned long long*)&cw->alive[s], (unsigned long long)(-removed));
         }
     }
+    end_push_last_block(p);
 }
 
 template <int K0, int K1, int K2>

@@ -203,7 +203,7 @@ __global__ void scan_blocks_kernel(long long* blocksum, int nb) {
 __global__ void scan_final_kernel(const int* hist, long long N, long long chunk, const long long* blocksum, long long* scan) {
     __shared__ long long sh[33];
     long long lo = blockIdx.x * chunk, hi = lo + chunk < N ? lo + chunk : N;
-    long long carry = blocksum[blockIdx.x];
+    long long carry = blocksum ? blocksum[blockIdx.x] : 0;
     for (long long t0 = lo; t0 < hi; t0 += blockDim.x) {
         long long i = t0 + threadIdx.x;
         long long v = i < hi ? hist[i] : 0;
@@ -489,14 +489,18 @@ int launch_sort(cpic_run* r, bool fused) {
         hist_kernel<<<(int)pblocks, 256, 0, r->stream>>>(p);
         CPIC_CHECK_LAUNCH();
     }
-    long long chunk = 4096;
+    // small grids: one block scans everything (4096 cells: 3 us in place of three launches)
+    constexpr long long SCAN_ONE = 16384;
+    long long chunk = N <= SCAN_ONE ? SCAN_ONE : 4096;
     while ((N + chunk - 1) / chunk > SCAN_THREADS) chunk *= 2;
     int nb = (int)((N + chunk - 1) / chunk);
-    scan_partial_kernel<<<nb, SCAN_THREADS, 0, r->stream>>>(r->hist, N, chunk, r->scan_blocks);
-    CPIC_CHECK_LAUNCH();
-    scan_blocks_kernel<<<1, SCAN_THREADS, 0, r->stream>>>(r->scan_blocks, nb);
-    CPIC_CHECK_LAUNCH();
-    scan_final_kernel<<<nb, SCAN_THREADS, 0, r->stream>>>(r->hist, N, chunk, r->scan_blocks, r->scan);
+    if (nb > 1) {
+        scan_partial_kernel<<<nb, SCAN_THREADS, 0, r->stream>>>(r->hist, N, chunk, r->scan_blocks);
+        CPIC_CHECK_LAUNCH();
+        scan_blocks_kernel<<<1, SCAN_THREADS, 0, r->stream>>>(r->scan_blocks, nb);
+        CPIC_CHECK_LAUNCH();
+    }
+    scan_final_kernel<<<nb, SCAN_THREADS, 0, r->stream>>>(r->hist, N, chunk, nb > 1 ? r->scan_blocks : nullptr, r->scan);
     CPIC_CHECK_LAUNCH();
     if (counted && fused) {
         long long most = 0;

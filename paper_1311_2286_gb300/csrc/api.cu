@@ -288,11 +288,24 @@ __global__ void set_count_kernel(DevCounters* ctr, int s, long long n) {
 // Loaded particles with a cell index outside the grid, an offset outside [0, 1) or a
 // non-finite velocity would make the mover read outside its vertex tables: they are
 // turned into dead slots and counted as dropped.
-__global__ void validate_load_kernel(int D, int n0, int n1, int n2, int* cell, const float* t, const float* v,
-                                     long long T, long long n, DevCounters* ctr, int s) {
+// COPY: the particles are read from the caller's device arrays (component stride n) and stored in the
+// same pass; else they are in place already. (Six device-to-device copies and a pass over the
+// result took 39 us of GPU time and as much on the host for a million 2D particles, 10 us so.)
+template <bool COPY>
+__global__ void __launch_bounds__(256) load_kernel(int D, int n0, int n1, int n2, const int* __restrict__ ucell,
+                                                   const float* __restrict__ ut, const float* __restrict__ uv, int* cell,
+                                                   float* pt, float* pv, long long T, long long n, DevCounters* ctr, int s) {
     long long bad = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        int w = cell[i];
+        float t[3], v[3];
+        for (int a = 0; a < D; ++a) t[a] = COPY ? ut[a * n + i] : pt[a * T + i];
+        for (int a = 0; a < 3; ++a) v[a] = COPY ? uv[a * n + i] : pv[a * T + i];
+        const int w = COPY ? ucell[i] : cell[i];
+        if (COPY) {
+            for (int a = 0; a < D; ++a) pt[a * T + i] = t[a];
+            for (int a = 0; a < 3; ++a) pv[a * T + i] = v[a];
+            cell[i] = w;
+        }
         if (w < 0) {
             ++bad;
             continue;
@@ -307,11 +320,8 @@ __global__ void validate_load_kernel(int D, int n0, int n1, int n2, int* cell, c
             c2 = w >> 20;
         }
         bool ok = c0 < n0 && c1 < n1 && (D == 2 || c2 < n2);
-        for (int a = 0; a < D; ++a) {
-            float x = t[a * T + i];
-            ok = ok && (x >= 0.0f) && (x < 1.0f);
-        }
-        for (int a = 0; a < 3; ++a) ok = ok && isfinite(v[a * T + i]);
+        for (int a = 0; a < D; ++a) ok = ok && (t[a] >= 0.0f) && (t[a] < 1.0f);
+        for (int a = 0; a < 3; ++a) ok = ok && isfinite(v[a]);
         if (!ok) {
             cell[i] = -1;
             ++bad;
@@ -398,6 +408,28 @@ __global__ void compact_scatter_kernel(int D, const int* cell, const float* t, c
         dst0 += total;
         __syncthreads();
     }
+}
+
+// one species' live particles into the caller's device arrays (component stride n)
+__global__ void __launch_bounds__(256) copy_out_kernel(int D, const int* __restrict__ cell, const float* __restrict__ t,
+                                                       const float* __restrict__ v, long long stride, long long n, int* ocell,
+                                                       float* ot, float* ov) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        ocell[i] = cell[i];
+        for (int a = 0; a < D; ++a) ot[a * n + i] = t[a * stride + i];
+        for (int a = 0; a < 3; ++a) ov[a * n + i] = v[a * stride + i];
+    }
+}
+
+// true for memory of the current device that a kernel may take in place of a copy
+bool device_memory(const void* p) {
+    cudaPointerAttributes at;
+    int dev = 0;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
 }
 
 // true for device, managed and page-locked host memory (a copy from it may stay in flight
@@ -989,7 +1021,8 @@ int cpic_load_particles(cpic_run* r, int sp, int64_t n, const int32_t* cell, con
     }
     int b = r->cur_host;
     long long base = r->pb.base[sp], T = r->pb.total;
-    if (n > 0) {
+    const bool direct = n > 0 && device_memory(cell) && device_memory(t) && device_memory(v);
+    if (n > 0 && !direct) {
         CPIC_CUDA(cudaMemcpyAsync(r->pb.cell[b] + base, cell, sizeof(int) * n, cudaMemcpyDefault, r->stream));
         for (int a = 0; a < r->D; ++a)
             CPIC_CUDA(cudaMemcpyAsync(r->pb.t[b] + a * T + base, t + a * n, sizeof(float) * n, cudaMemcpyDefault, r->stream));
@@ -1000,14 +1033,15 @@ int cpic_load_particles(cpic_run* r, int sp, int64_t n, const int32_t* cell, con
     CPIC_CHECK_LAUNCH();
     if (n > 0) {
         long long blocks = (n + 255) / 256;
-        if (blocks > 4LL * device_sm_count()) blocks = 4LL * device_sm_count();
-        validate_load_kernel<<<(int)blocks, 256, 0, r->stream>>>(r->D, r->n[0], r->n[1], r->n[2], r->pb.cell[b] + base,
-                                                                 r->pb.t[b] + base, r->pb.v[b] + base, T, n, r->ctr, sp);
+        if (blocks > 8LL * device_sm_count()) blocks = 8LL * device_sm_count();
+        auto kernel = direct ? load_kernel<true> : load_kernel<false>;
+        kernel<<<(int)blocks, 256, 0, r->stream>>>(r->D, r->n[0], r->n[1], r->n[2], cell, t, v, r->pb.cell[b] + base,
+                                                   r->pb.t[b] + base, r->pb.v[b] + base, T, n, r->ctr, sp);
         CPIC_CHECK_LAUNCH();
     }
     // copies from pageable host memory must be complete before the caller may free or reuse
     // it; device and page-locked inputs stay stream-ordered (asynchronous)
-    if (n > 0 && !(stream_ordered_source(cell) && stream_ordered_source(t) && stream_ordered_source(v)))
+    if (n > 0 && !direct && !(stream_ordered_source(cell) && stream_ordered_source(t) && stream_ordered_source(v)))
         CPIC_CUDA(cudaStreamSynchronize(r->stream));
     return CPIC_OK;
 }
@@ -1074,7 +1108,15 @@ int cpic_get_particles(cpic_run* r, int sp, int64_t room, int64_t* n, int32_t* c
             return CPIC_ERR_STATE;
         }
     }
-    // one copy per array into the caller's buffers (host or device)
+    // into the caller's buffers: one pass where they are on this device, else one copy per array
+    if (device_memory(cell) && device_memory(t) && device_memory(v)) {
+        long long nb = (live + 255) / 256;
+        if (nb > 8LL * device_sm_count()) nb = 8LL * device_sm_count();
+        copy_out_kernel<<<(int)nb, 256, 0, r->stream>>>(r->D, src_c, src_t, src_v, stride, live, cell, t, v);
+        CPIC_CHECK_LAUNCH();
+        CPIC_CUDA(cudaStreamSynchronize(r->stream));
+        return CPIC_OK;
+    }
     CPIC_CUDA(cudaMemcpyAsync(cell, src_c, sizeof(int) * live, cudaMemcpyDefault, r->stream));
     for (int a = 0; a < r->D; ++a)
         CPIC_CUDA(cudaMemcpyAsync(t + a * live, src_t + a * stride, sizeof(float) * live, cudaMemcpyDefault, r->stream));

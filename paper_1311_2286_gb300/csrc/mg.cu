@@ -587,6 +587,33 @@ __global__ void smooth_kernel(LV<float> L, const float* __restrict__ dinv, int c
     smooth_at<D, NPT>(L, dinv, q);
 }
 
+// The first two colour sweeps of a 3D two-colour level, from x = 0, in one pass: the first colour
+// is b / diag, so the second reads its neighbours' b and 1 / diag in place of their x (the same
+// products in the same order). A thread takes the two cells of a pair along axis 0 (n[0] is even
+// on a level that coarsens). Bound by L2: a colour's sweep touches every sector of the operator
+// and uses half of it, so two sweeps in one pass read it once. 128^3 and the 64^3 level below:
+// 16.1 us a V-cycle, 21 us as a memset and two sweeps each.
+__global__ void __launch_bounds__(256) first_sweeps3_kernel(const __grid_constant__ LV<float> L) {
+    const int m = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 8 + threadIdx.y, k = blockIdx.z;
+    const int n0 = L.n[0], n1 = L.n[1], pl = n0 * n1, nc = L.ncell;
+    if (2 * m >= n0 || j >= n1) return;
+    const int c = 2 * m + n0 * (j + n1 * k), odd = (j + k) & 1;  // the first colour is cell c + odd
+    const float2 b = *reinterpret_cast<const float2*>(L.b + c), d = __ldg(reinterpret_cast<const float2*>(L.dinv + c));
+    const float x0 = (odd ? b.y : b.x) * (odd ? d.y : d.x);
+    const int e = c + 1 - odd, i = 2 * m + 1 - odd;  // the second colour's cell
+    auto first = [&](int q) { return L.b[q] * __ldg(L.dinv + q); };
+    // beyond a closed face the stencil entry is zero: any neighbour will do
+    float s = 0.0f;
+    s += __ldg(L.A + nc + e) * (odd ? first(e + (i > 0 ? -1 : n0 - 1)) : x0);
+    s += __ldg(L.A + 2 * nc + e) * (odd ? x0 : first(e + (i < n0 - 1 ? 1 : 1 - n0)));
+    s += __ldg(L.A + 3 * nc + e) * first(e + (j > 0 ? -1 : n1 - 1) * n0);
+    s += __ldg(L.A + 4 * nc + e) * first(e + (j < n1 - 1 ? 1 : 1 - n1) * n0);
+    s += __ldg(L.A + 5 * nc + e) * first(e + (k > 0 ? -1 : L.n[2] - 1) * pl);
+    s += __ldg(L.A + 6 * nc + e) * first(e + (k < L.n[2] - 1 ? 1 : 1 - L.n[2]) * pl);
+    const float x1 = ((odd ? b.x : b.y) - s) * (odd ? d.x : d.y);
+    *reinterpret_cast<float2*>(L.x + c) = odd ? make_float2(x1, x0) : make_float2(x0, x1);
+}
+
 template <int D, int NPT>
 __global__ void __launch_bounds__(256) restrict_kernel(LV<float> F, LV<float> Cl) {
     // one thread per fine cell (block RB_X x RB_Y x RB_Z fine cells): its residual goes to
@@ -2281,7 +2308,8 @@ int enqueue_vcycle(cpic_run* r, const LVSet& S) {
             }
             return CPIC_OK;
         }
-        if (top > 0) CPIC_CUDA(cudaMemsetAsync(r->lev[0].x32, 0, sizeof(float) * r->lev[0].ncell, st));
+        const bool first = D == 3 && NPT == 7 && !S.line && nu1 > 0;  // the first two sweeps in one pass
+        if (top > 0 && !first) CPIC_CUDA(cudaMemsetAsync(r->lev[0].x32, 0, sizeof(float) * r->lev[0].ncell, st));
         auto smooth = [&](int l, int col) -> int {
             const LV<float>& L = S.l[l];
             int d[3] = {L.n[0] / 2, Col<D, NPT>::parity ? L.n[1] : L.n[1] / 2,
@@ -2311,6 +2339,12 @@ int enqueue_vcycle(cpic_run* r, const LVSet& S) {
             for (int it = 0; it < nu1; ++it) {
                 if (S.line) {
                     if (int e = line_smooth(l, false)) return e;
+                    continue;
+                }
+                if (first && it == 0) {
+                    const LV<float>& L = S.l[l];
+                    first_sweeps3_kernel<<<cell_grid(L.n[0] / 2, L.n[1], L.n[2]), kCellBlock, 0, st>>>(L);
+                    CPIC_CHECK_LAUNCH();
                     continue;
                 }
                 for (int col = 0; col < S.l[l].ncol; ++col)

@@ -273,8 +273,9 @@ int cpic_load_maxwellian(cpic_run* run, int sp, int64_t n, double vth, const dou
 int cpic_initialize(cpic_run* run);
 /* nsteps full PIC steps (Sec. II cycle): vertex field, push (+ deposit), injection, sort
  * every sort_interval steps, charge -> RHS, multigrid solve to mg_rtol, diagnostics.
- * When the push is the direct 3D kernel or the 2D kernel, a sort takes its histogram from
- * the step's push and injection and leaves its reordering to the next push, which reads
+ * When the push is the direct 3D kernel or the 2D kernel, the step's push and injection
+ * count the cells and number the particles in each, so that a sort is a scan and a look-up of
+ * every particle's slot; it leaves its reordering to the next push, which reads
  * each sorted slot's particle through the sort's index; every other call that touches the
  * particles (reads, loads, injection, checkpoints, another push kernel) carries out such a
  * pending order first, so the particles are always seen in sorted slot order. */
@@ -319,6 +320,9 @@ int cpic_solve_field(cpic_run* run, double rtol, int max_cycles, int* cycles, do
  *                         the V-cycles on the 3D shell, and it converges where point smoothing
  *                         alone stalls on strongly anisotropic cells). The stopping test and
  *                         the result's accuracy are the same; mg_cycles counts V-cycles.
+ *                         A grid whose levels all fit one CTA's shared memory (point
+ *                         smoothing, bilinear prolongation) runs the whole solve as one
+ *                         kernel, with the same operations.
  * Invalidates the run's captured step graphs. CPIC_ERR_INVALID for another value. */
 #define CPIC_SOLVER_MG 0
 #define CPIC_SOLVER_BICGSTAB 1

@@ -64,7 +64,7 @@ struct DevCounters {
     double float_cpsi;
     // 1: a sort's new order is pending: slot i of the other buffer's cell array holds the
     // index (in the current buffer) of the particle that belongs in slot i, and the counts
-    // are already the sorted ones; the next fused 3D push reads through it and the step's
+    // are already the sorted ones; the next push reads through it and the step's
     // finalisation flips the buffers (see launch_sort)
     int perm;
 };
@@ -147,7 +147,8 @@ struct Level {
     float* x32;       // FP32 correction
     float* b32;       // FP32 residual / right-hand side of the correction
     float* dinv32;    // FP32 inverse diagonal (Gauss-Seidel)
-    float* lw;        // line-relaxation work [2][ncell] (eliminated upper diagonal, 2nd solve)
+    float* lw;        // line-relaxation work [2][ncell] (eliminated upper diagonal, 2nd solve); the
+                      // fused 2D levels' second x buffer
     double* pw;       // operator-induced prolongation weights [D][ncell] of this (fine) level
     float* pw32;      // their FP32 copy (the V-cycle's prolongation)
 };
@@ -210,7 +211,8 @@ struct cpic_run {
     int cluster_nd;              // its split levels
     int slab_cs;                 // largest cluster of the 3D V-cycle's cluster part (0: none)
     bool order_pending;          // a fused sort's order may be pending on the device (DevCounters::perm)
-    bool count_hist;             // this step's direct 3D push and injection build the sort's histogram
+    bool count_hist;             // this step's push and injection count the cells (hist) and number
+                                 // the particles in them (prank)
     int dense_m;                 // coarsest unknowns (+1 row when singular)
     bool singular;
     double sumJ;                 // sum of finest J_c (singular projection)
@@ -233,10 +235,11 @@ struct cpic_run {
     int push_chunk;              // push kernel: particles per block chunk (0: one wave)
     int push_tile;               // push kernel: shared-memory deposit tile (1) or direct (0)
     cpic::KrylovState* kry;      // device scalars of the Krylov solve
-    double* kv;                  // Krylov vectors, FP64 [5][ncell]: r, r_hat, p, v, s
+    double* kv;                  // Krylov vectors: r, r_hat (FP64), p, v, s (FP32); with the cluster
+                                 // solver, which needs none, its operator as pairs of floats
     float* ph32;                 // preconditioned direction p_hat (FP32)
     // sort scratch
-    int* hist;                   // [nsp][ncell] counts -> cursors
+    int* hist;                   // [nsp][ncell] counts (-> cursors of the rank pass)
     int* prank;                  // [slot] a particle's number among its cell's (counted steps)
     long long* scan;             // [nsp*ncell + 1] exclusive prefix
     long long* scan_blocks;      // block partials

@@ -246,20 +246,6 @@ __device__ __forceinline__ void smooth_at(const LV<R>& L, const R* dinv, const i
     L.x[c] = (L.b[c] - stencil_sum<D, NPT, 1>(L, c, q)) * dinv[c];
 }
 
-template <int D, int NPT, typename R>
-__device__ __forceinline__ void restrict_at(const LV<R>& F, const LV<R>& Cl, const int* qc) {
-    R acc = R(0);
-#pragma unroll
-    for (int ch = 0; ch < (D == 2 ? 4 : 8); ++ch) {
-        int q[3] = {2 * qc[0] + (ch & 1), 2 * qc[1] + ((ch >> 1) & 1), D == 3 ? 2 * qc[2] + ((ch >> 2) & 1) : 0};
-        int f = q[0] + F.n[0] * (q[1] + F.n[1] * q[2]);
-        acc += F.b[f] - stencil_sum<D, NPT, 0>(F, f, q);
-    }
-    int C = qc[0] + Cl.n[0] * (qc[1] + Cl.n[1] * qc[2]);
-    Cl.b[C] = acc;
-    Cl.x[C] = R(0);
-}
-
 // Prolongation x_f += sum over the 2^D parents of w * x_parent: per axis the fine cell's own
 // parent (weight own, 3/4 when bilinear) and the parent on the fine cell's side (1 - own,
 // with the correction's ghost rules: periodic wrap, or else the boundary parent itself, its
@@ -618,7 +604,7 @@ template <int D, int NPT>
 __global__ void __launch_bounds__(256) restrict_kernel(LV<float> F, LV<float> Cl) {
     // one thread per fine cell (block RB_X x RB_Y x RB_Z fine cells): its residual goes to
     // shared memory, then one thread per coarse cell of the block sums its 2^D children in
-    // restrict_at's order (children ch = 0 .. 2^D - 1, axis 0 fastest)
+    // the children's order: ch = 0 .. 2^D - 1, axis 0 fastest
     constexpr int BX = 32, BY = D == 3 ? 4 : 8, BZ = D == 3 ? 2 : 1;
     __shared__ float rs[BX * BY * BZ];
     const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
@@ -1125,7 +1111,6 @@ constexpr size_t SL_SMEM_MAX = 216 * 1024;
 struct SlabPlan {
     int cs;          // CTAs
     int first, ns;   // split levels first .. first + ns - 1; the one-CTA levels follow
-    int rmax[SL_MAX];  // most planes of a CTA
     int oa[SL_MAX], od[SL_MAX], ob[SL_MAX], ox[SL_MAX];  // shared offsets (words)
     int ocoarse;     // of the one-CTA levels
     int odense;      // of the dense inverse (0: global)
@@ -2199,7 +2184,6 @@ bool plan_slabs(const LVSet& S, int cs_max, SlabPlan* P, size_t* smem) {
         for (int t = 0; t < ns; ++t) {
             const LV<float>& L = S.l[first + t];
             const size_t plane = (size_t)L.n[0] * L.n[1], R = (size_t)((planes + cs - 1) / cs) << (ns - t);
-            P->rmax[t] = (int)R;
             P->oa[t] = (int)off, off += 7 * R * plane;
             P->od[t] = (int)off, off += R * plane;
             P->ob[t] = (int)off, off += R * plane;

@@ -6,7 +6,9 @@
 // dead slots away: histogram (warp-aggregated atomics) -> exclusive scan over
 // [species][cell] -> rank (each live particle's slot in the other buffer; one atomic per cell
 // group reserves consecutive slots; the order inside a cell is unspecified) -> gather of the
-// particle data into the other buffer in slot order -> live counts.
+// particle data into the other buffer in slot order -> live counts. At the end of a step whose
+// push and injection numbered the particles of each cell, only the scan and a look-up of the
+// slot are left (place_kernel), and the gather is the next push's.
 #include "particles.cuh"
 
 namespace cpic {
@@ -374,9 +376,12 @@ __global__ void __launch_bounds__(256) gather_kernel(SortParams p) {
 // After a counted step (the push and the injection have numbered the particles of each cell): a
 // particle's slot is its cell's start plus its number. The slot receives the particle's
 // source index, as in the rank pass; the last block to finish makes the live counts the sorted
-// ones and leaves the order pending (see launch_sort). Four particles a thread with 16-byte
-// loads. 64M particles on 128^3 cells: 170 us, against 537 us for the rank pass, which counts
-// every chunk's cells again (255 against 372 us on 512 x 1024, sorted every other step); the returned counts cost the push 5 %.
+// ones and leaves the order pending: the next push reads slot i's particle from the index
+// stored in the other buffer, writes it to slot i there, and the step's finalisation flips the
+// buffers. Four particles a thread with 16-byte loads (a species' slots start at a multiple of
+// 32). 64M particles on 128^3 cells: 170 us, against 537 us for the rank pass, which counts
+// every chunk's cells again (255 against 372 us on 512 x 1024, sorted every other step); the
+// returned counts cost the push 5 %.
 template <int D>
 __global__ void __launch_bounds__(256) place_kernel(SortParams p, const int* __restrict__ rank) {
     __shared__ bool last;
@@ -414,19 +419,6 @@ __global__ void __launch_bounds__(256) place_kernel(SortParams p, const int* __r
     if (!last || threadIdx.x != 0) return;
     __threadfence();
     *p.ticket = 0;
-    for (int sp = 0; sp < p.nsp; ++sp) {
-        const long long cnt = p.scan[(long long)(sp + 1) * p.ncell] - p.scan[(long long)sp * p.ncell];
-        p.ctr->count[sp] = cnt;
-        p.ctr->alive[sp] = cnt;
-    }
-    p.ctr->perm = 1;
-}
-
-// Fused sort: the live counts become the sorted ones and the order is left pending; the next
-// push reads slot i's particle from the index the rank pass stored in the other buffer, writes
-// it to slot i there, and the step's finalisation flips the buffers.
-__global__ void sort_fused_finish_kernel(SortParams p) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     for (int sp = 0; sp < p.nsp; ++sp) {
         const long long cnt = p.scan[(long long)(sp + 1) * p.ncell] - p.scan[(long long)sp * p.ncell];
         p.ctr->count[sp] = cnt;
@@ -482,9 +474,12 @@ int launch_sort(cpic_run* r, bool fused) {
     long long pblocks = (tot + 255) / 256;
     if (pblocks > 8LL * device_sm_count()) pblocks = 8LL * device_sm_count();
     if (pblocks < 1) pblocks = 1;
-    const bool counted = r->count_hist;  // the step's push and injection counted the cells
+    if (fused && !r->count_hist) {
+        set_error("the step has not numbered its particles");
+        return CPIC_ERR_STATE;
+    }
     r->count_hist = false;
-    if (!counted) {
+    if (!fused) {
         CPIC_CUDA(cudaMemsetAsync(r->hist, 0, sizeof(int) * N, r->stream));
         hist_kernel<<<(int)pblocks, 256, 0, r->stream>>>(p);
         CPIC_CHECK_LAUNCH();
@@ -502,7 +497,7 @@ int launch_sort(cpic_run* r, bool fused) {
     }
     scan_final_kernel<<<nb, SCAN_THREADS, 0, r->stream>>>(r->hist, N, chunk, nb > 1 ? r->scan_blocks : nullptr, r->scan);
     CPIC_CHECK_LAUNCH();
-    if (counted && fused) {
+    if (fused) {
         long long most = 0;
         for (int s = 0; s < p.nsp; ++s) most = r->pb.capacity[s] > most ? r->pb.capacity[s] : most;
         long long nb = (most + 1023) / 1024, cap = 8LL * device_sm_count() / p.nsp;
@@ -520,12 +515,6 @@ int launch_sort(cpic_run* r, bool fused) {
     else
         rank_kernel<3><<<(int)pblocks, 256, 0, r->stream>>>(p);
     CPIC_CHECK_LAUNCH();
-    if (fused) {
-        sort_fused_finish_kernel<<<1, 32, 0, r->stream>>>(p);
-        CPIC_CHECK_LAUNCH();
-        r->order_pending = true;
-        return CPIC_OK;
-    }
     return launch_gather(r, p);
 }
 

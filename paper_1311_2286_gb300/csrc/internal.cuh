@@ -209,6 +209,7 @@ struct cpic_run {
     cudaStream_t capture_stream;
     int cluster_cs;              // cluster size of the cluster solver (0: not applicable)
     int cluster_nd;              // its split levels
+    bool cluster_class;          // V-cycles are the outer iteration, also where no cluster layout fits
     int slab_cs;                 // largest cluster of the 3D V-cycle's cluster part (0: none)
     bool order_pending;          // a fused sort's order may be pending on the device (DevCounters::perm)
     bool count_hist;             // this step's push and injection count the cells (hist) and number

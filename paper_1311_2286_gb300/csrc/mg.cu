@@ -2449,7 +2449,7 @@ int enqueue_bicg_iteration(cpic_run* r, const LVSet& S, double rtol, int max_cyc
 
 // the one-CTA solve's shared memory, or 0 where it does not apply
 size_t cta_solve_bytes(const cpic_run* r, const LVSet& S, CtaSolve* P) {
-    if (r->solver != CPIC_SOLVER_BICGSTAB || r->cluster_cs || S.first_cta != 0 || S.nl < 2 || S.line || S.l[0].pw ||
+    if (r->solver != CPIC_SOLVER_BICGSTAB || r->cluster_class || S.first_cta != 0 || S.nl < 2 || S.line || S.l[0].pw ||
         r->mg_coarse == CPIC_MG_COARSE_GALERKIN)
         return 0;
     size_t f = (cta_words(S, 0) + 3) & ~size_t(3);
@@ -2489,7 +2489,7 @@ int enqueue_cta_solve(cpic_run* r, const LVSet& S, CtaSolve P, size_t smem, doub
                   : (face ? launch_cta_solve<3, 7, 19>(r, S, P, smem) : launch_cta_solve<3, 19, 19>(r, S, P, smem));
 }
 
-bool use_krylov(const cpic_run* r) { return r->solver == CPIC_SOLVER_BICGSTAB && !r->cluster_cs; }
+bool use_krylov(const cpic_run* r) { return r->solver == CPIC_SOLVER_BICGSTAB && !r->cluster_class; }
 
 // right-hand side (and its projection); resets the solve counters
 int enqueue_prologue(cpic_run* r, bool fold) {

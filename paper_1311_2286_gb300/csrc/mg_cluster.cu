@@ -616,11 +616,14 @@ __global__ void split_operator_kernel(const double* A, float* out, int n0, int n
     }
 }
 
-// Which runs iterate V-cycles on the cluster: 2D, no cross terms, the default multigrid
-// components, an even first axis on every level, and a finest level that 16 or 8 CTAs can
-// split into even slabs of at least four rows within 200 KB of eight words a cell. (Other runs
-// take the kernel chain's outer iteration; the two stop at the same tolerance, but at
-// different points below it.)
+// Which runs iterate V-cycles: 2D, no cross terms, the default multigrid components, an even
+// first axis on every level, and a finest level that 16 or 8 CTAs can split into even slabs of
+// at least four rows within 200 KB of eight words a cell. (Other runs take the kernel chain's
+// outer iteration; the two stop at the same tolerance, but at different points below it.) Nearly
+// all of them run on the cluster; where no layout of the halo slabs fits (192 x 128, 256 x 64
+// and other grids long in axis 0: the halo rows outweigh the slab) the same iteration runs on
+// the kernels per level: a 256 x 128 cylinder step takes 1276 us for its 30 V-cycles (1900 us in
+// one cluster with slabs without halos, which fit).
 bool cluster_takes(const cpic_run* r) {
     if (r->D != 2 || r->lev[0].cross || r->nlevels < 2 || r->nlevels > CL_MAX_LEVELS) return false;
     if (r->mg_coarse != CPIC_MG_COARSE_REDISCRETIZED || r->mg_smoother != CPIC_MG_SMOOTH_POINT ||
@@ -745,8 +748,8 @@ void cluster_config(const ClusterPlan& plan, cudaLaunchConfig_t* cfg, cudaLaunch
 // number of split levels (the cheapest that the device can co-schedule).
 int mg_cluster_prepare(cpic_run* r) {
     r->cluster_cs = 0;
-    if (getenv("CPIC_NO_CLUSTER_SOLVER")) return CPIC_OK;
-    if (!cluster_takes(r)) return CPIC_OK;
+    r->cluster_class = !getenv("CPIC_NO_CLUSTER_SOLVER") && cluster_takes(r);
+    if (!r->cluster_class) return CPIC_OK;
     // the attributes are per function, shared by every run of the process: raise them to the
     // device's maximum once (they bound launches, they do not change occupancy)
     int dev = 0, optin = 0;

@@ -1,6 +1,8 @@
 // C ABI of include/cpic.h: validation, device-memory planning (one arena per run), the PIC
 // cycle's orchestration on the run's stream, and data transfer. All arithmetic of the
 // method runs in the kernels of geometry.cu, fields.cu, push.cu, inject.cu, sort.cu, mg.cu.
+#include <cuda.h>
+#include <stdint.h>
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -421,15 +423,32 @@ __global__ void __launch_bounds__(256) copy_out_kernel(int D, const int* __restr
     }
 }
 
-// true for memory of the current device that a kernel may take in place of a copy
-bool device_memory(const void* p) {
+// true for an array of the current device that a kernel may take in place of a copy: aligned to its
+// words and inside one allocation. Every other array goes to the copies, which take any byte
+// address and refuse a range that leaves its allocation.
+bool device_memory(const void* p, size_t bytes) {
     cudaPointerAttributes at;
     int dev = 0;
+    if ((uintptr_t)p % 4) return false;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
+    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+    void* entry = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &entry, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    if (((CUresult(*)(CUdeviceptr*, size_t*, CUdeviceptr))entry)(&base, &size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    return (CUdeviceptr)p - base <= size && bytes <= size - ((CUdeviceptr)p - base);
+}
+bool device_memory(int D, long long n, const void* cell, const void* t, const void* v) {
+    return device_memory(cell, 4 * (size_t)n) && device_memory(t, 4 * (size_t)n * D) && device_memory(v, 12 * (size_t)n);
 }
 
 // true for device, managed and page-locked host memory (a copy from it may stay in flight
@@ -1021,7 +1040,7 @@ int cpic_load_particles(cpic_run* r, int sp, int64_t n, const int32_t* cell, con
     }
     int b = r->cur_host;
     long long base = r->pb.base[sp], T = r->pb.total;
-    const bool direct = n > 0 && device_memory(cell) && device_memory(t) && device_memory(v);
+    const bool direct = n > 0 && device_memory(r->D, n, cell, t, v);
     if (n > 0 && !direct) {
         CPIC_CUDA(cudaMemcpyAsync(r->pb.cell[b] + base, cell, sizeof(int) * n, cudaMemcpyDefault, r->stream));
         for (int a = 0; a < r->D; ++a)
@@ -1109,7 +1128,7 @@ int cpic_get_particles(cpic_run* r, int sp, int64_t room, int64_t* n, int32_t* c
         }
     }
     // into the caller's buffers: one pass where they are on this device, else one copy per array
-    if (device_memory(cell) && device_memory(t) && device_memory(v)) {
+    if (device_memory(r->D, live, cell, t, v)) {
         long long nb = (live + 255) / 256;
         if (nb > 8LL * device_sm_count()) nb = 8LL * device_sm_count();
         copy_out_kernel<<<(int)nb, 256, 0, r->stream>>>(r->D, src_c, src_t, src_v, stride, live, cell, t, v);

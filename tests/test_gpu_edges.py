@@ -217,3 +217,39 @@ def test_drifting_inversion_over_the_drifts(cpic, drift):
     assert np.sum(~ok) <= 1
     np.testing.assert_allclose(v[:, ok], v32[:, ok], rtol=2e-6, atol=2e-6 * vth)
     np.testing.assert_allclose(t[:, ok], t32[:, ok], atol=1e-5)
+
+
+@pytest.mark.parametrize("shifted", [0, 1, 2])
+def test_device_arrays_off_their_words_are_copied(cpic, shifted):
+    """A device array at an odd byte address (cell, t or v) loads and reads as it does at a word."""
+    torch = pytest.importorskip("torch")
+    n = 1000
+    w = wl.cylinder(16, 32, npart_per_species=n)
+    arrays = [np.ascontiguousarray(x) for x in (w.particles[0].cell, w.particles[0].t, w.particles[0].v)]
+    run = cpic.Run(cpic.config_from_workload(w))
+    run.set_map_vertices(w.vertices)
+
+    def room(k, nbytes):
+        at = 2 if k == shifted else 0
+        return torch.zeros(nbytes + 64, dtype=torch.uint8, device="cuda")[at:at + nbytes]
+
+    bufs = [room(k, x.nbytes) for k, x in enumerate(arrays)]
+    for b, x in zip(bufs, arrays):
+        b.copy_(torch.from_numpy(x.reshape(-1).view(np.uint8)))
+    torch.cuda.synchronize()
+    ptrs = [ctypes.c_void_p(b.data_ptr()) for b in bufs]
+    assert ptrs[shifted].value % 4 == 2
+    cpic.check(cpic.load().cpic_load_particles(run.h, 0, n, *ptrs))
+    run.synchronize()
+    for a, b in zip(run.particles(0), arrays):
+        assert np.array_equal(a.reshape(-1), b.reshape(-1))
+    for b in bufs:
+        b.zero_()
+    torch.cuda.synchronize()
+    m = ctypes.c_int64()
+    cpic.check(cpic.load().cpic_get_particles(run.h, 0, n, ctypes.byref(m), *ptrs))
+    run.synchronize()
+    assert m.value == n
+    for b, x in zip(bufs, arrays):
+        assert np.array_equal(b.cpu().numpy(), x.reshape(-1).view(np.uint8))
+    run.close()

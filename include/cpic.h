@@ -310,7 +310,8 @@ int cpic_sort(cpic_run* run);
 int cpic_solve_field(cpic_run* run, double rtol, int max_cycles, int* cycles, double* residual);
 
 /* Outer iteration of the field solve on the kernel-chain path (3D runs, and 2D runs that the
- * one-cluster solver does not take; the cluster solver always iterates V-cycles):
+ * one-cluster solver does not take; that one always iterates V-cycles, also on those of its
+ * grids that need the kernels per level):
  *   CPIC_SOLVER_MG        x += V-cycle(b - M x) until ||r||/||b|| <= rtol (Sec. II.B.3's
  *                         multigrid iteration);
  *   CPIC_SOLVER_BICGSTAB  BiCGStab (van der Vorst, SIAM J. Sci. Stat. Comput. 13, 1992) on
@@ -341,8 +342,8 @@ int cpic_set_solver(cpic_run* run, int solver);
  * colour-ordered point Gauss-Seidel) or CPIC_MG_SMOOTH_LINE (alternating zebra line
  * Gauss-Seidel: every line of cells along axis 0, then along axis 1 (then axis 2), solved
  * exactly, cyclic on a periodic axis). Any non-default choice runs the solve on the kernel
- * chain (not the one-cluster solver). CPIC_ERR_INVALID for an unknown value. Synchronous when the map is already set (the hierarchy is rebuilt);
- * invalidates captured step graphs. */
+ * chain (not the one-cluster solver). CPIC_ERR_INVALID for an unknown value. Synchronous when
+ * the map is already set (the hierarchy is rebuilt); invalidates captured step graphs. */
 #define CPIC_MG_COARSE_REDISCRETIZED 0
 #define CPIC_MG_COARSE_GALERKIN 1
 #define CPIC_MG_INTERP_BILINEAR 0

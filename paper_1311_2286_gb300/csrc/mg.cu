@@ -1684,6 +1684,7 @@ __global__ void __launch_bounds__(CS_THREADS, 1) cta_solve_kernel(const __grid_c
         if (P.odense) load.copy(sm + P.odense, S.dense_inv, (unsigned)((mm * mm * 4 + 15) & ~15));
         load.arrive();
     }
+    __syncthreads();  // the barrier is initialised before any other thread waits on it
     for (int c = tid; c < n; c += CS_THREADS) phi[c] = P.phi[c];
     bulk_wait(&bar);
     __syncthreads();

@@ -354,7 +354,10 @@ int cpic_set_multigrid(cpic_run* run, int coarse, int interpolation, int smoothe
 
 /* ---------------------------------------------------------------- data out / in */
 
-int cpic_get_diag(cpic_run* run, cpic_diag* out);              /* synchronises */
+/* Synchronises. CPIC_ERR_TIMEOUT (with *out filled in) when a solver kernel's bounded wait for its
+ * data ran out in a step or solve since the last cpic_initialize or cpic_solve_field: the
+ * potential is not valid from there on. cpic_solve_field returns the same of its own solve. */
+int cpic_get_diag(cpic_run* run, cpic_diag* out);
 int cpic_get_phi(cpic_run* run, double* phi);                  /* host or device, cells */
 int cpic_set_phi(cpic_run* run, const double* phi);            /* host or device, cells */
 int cpic_get_charge(cpic_run* run, int sp, int64_t* counts);   /* host or device, cells;

@@ -47,6 +47,11 @@ int cuda_fail(cudaError_t e, const char* what, const char* file, int line) {
     return e == cudaErrorMemoryAllocation ? CPIC_ERR_OOM : CPIC_ERR_CUDA;
 }
 
+int wait_ran_out() {
+    set_error("field solve: a kernel's wait for its data ran out; the potential is not valid");
+    return CPIC_ERR_TIMEOUT;
+}
+
 namespace {
 
 // ------------------------------------------------------------------ memory planning
@@ -1233,7 +1238,13 @@ int cpic_set_floating(cpic_run* r, int face, double charge0) {
     }
     CPIC_CUDA(cudaMemsetAsync(r->lev[0].x, 0, sizeof(double) * r->ncell, r->stream));
     invalidate_graphs(r);
+    int solved = 0;  // psi's solve
+    CPIC_CUDA(cudaMemcpyAsync(&solved, &r->ctr->mg_converged, sizeof(int), cudaMemcpyDeviceToHost, r->stream));
     CPIC_CUDA(cudaStreamSynchronize(r->stream));
+    if (solved == MG_WAIT_RAN_OUT) {
+        r->floating_face = -1;
+        return wait_ran_out();
+    }
     return CPIC_OK;
 }
 
@@ -1283,6 +1294,7 @@ int cpic_initialize(cpic_run* r) {
     CHECK_MAP(r);
     int st = launch_deposit(r);
     if (st) return st;
+    CPIC_CUDA(cudaMemsetAsync(&r->ctr->mg_converged, 0, sizeof(int), r->stream));
     st = mg_solve(r, r->cfg.mg_rtol, r->cfg.mg_max_cycles, true, nullptr, nullptr);
     if (st) return st;
     st = launch_vertex_field(r);
@@ -1367,6 +1379,7 @@ int cpic_solve_field(cpic_run* r, double rtol, int max_cycles, int* cycles, doub
     }
     int c = 0;
     double res = 0.0;
+    CPIC_CUDA(cudaMemsetAsync(&r->ctr->mg_converged, 0, sizeof(int), r->stream));
     int st = mg_solve(r, rtol, max_cycles, false, &c, &res);
     if (cycles) *cycles = c;
     if (residual) *residual = res;
@@ -1400,7 +1413,7 @@ int cpic_get_diag(cpic_run* r, cpic_diag* out) {
     out->pc_face_only = r->pc_face_only;
     out->object_potential = r->floating_face >= 0 ? h.object_potential : 0.0;
     out->object_charge = r->floating_face >= 0 ? h.object_charge : 0.0;
-    return CPIC_OK;
+    return h.mg_converged == MG_WAIT_RAN_OUT ? wait_ran_out() : CPIC_OK;
 }
 
 int cpic_get_phi(cpic_run* r, double* phi) {

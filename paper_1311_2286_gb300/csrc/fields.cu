@@ -156,7 +156,7 @@ __device__ __forceinline__ void reset_solve(const SolveReset& z) {
     *z.done = 0;
     *z.ticket = 0;
     z.ctr->mg_cycles = 0;
-    z.ctr->mg_converged = 0;
+    if (z.ctr->mg_converged != MG_WAIT_RAN_OUT) z.ctr->mg_converged = 0;
 }
 
 __global__ void rhs_kernel(RhsParams p, double* b, SolveReset z) {

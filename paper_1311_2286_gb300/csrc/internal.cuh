@@ -23,6 +23,7 @@ constexpr int DENSE_MAX = 512;      // coarsest level solved densely (inverse) u
 // ---------------------------------------------------------------- error handling
 void set_error(const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what, const char* file, int line);
+int wait_ran_out();  // CPIC_ERR_TIMEOUT of a field solve
 #define CPIC_CUDA(call)                                                      \
     do {                                                                     \
         cudaError_t e_ = (call);                                             \
@@ -40,6 +41,7 @@ void add_launches(long long n);  // kernels launched by a graph replay
     } while (0)
 
 // ---------------------------------------------------------------- device-side run state
+constexpr int MG_WAIT_RAN_OUT = -1;  // DevCounters::mg_converged: a solver kernel's data did not arrive
 // Counters written by kernels (one struct in device memory per run).
 struct DevCounters {
     long long count[CPIC_MAX_SPECIES];     // occupied slots (live + dead until the next sort)
@@ -56,7 +58,7 @@ struct DevCounters {
     double mg_residual;
     double mg_bnorm;
     int mg_cycles;
-    int mg_converged;
+    int mg_converged;  // of the last solve; MG_WAIT_RAN_OUT stays until cpic_solve_field or cpic_initialize
     // floating conductor (cpic_set_floating): its potential and charge after the last solve,
     // and the flux sum of the unit-potential solution (set once)
     double object_potential;
@@ -68,6 +70,10 @@ struct DevCounters {
     // finalisation flips the buffers (see launch_sort)
     int perm;
 };
+
+__device__ __forceinline__ void set_converged(DevCounters* ctr) {
+    if (ctr->mg_converged != MG_WAIT_RAN_OUT) ctr->mg_converged = 1;
+}
 
 // Scalars and reduction partials of the Krylov solve (device).
 // blocks of the operator passes over the finest level (the FP64 residual, the Krylov

@@ -98,6 +98,7 @@ struct LVSet {
     int first_cta;  // first level solved inside one CTA
     int line;       // 1: alternating zebra line relaxation (2D) instead of point smoothing
     LV<float> l[MAX_LEVELS];
+    int* status;    // DevCounters::mg_converged, for a wait that ran out
     const float* dense_inv;  // transposed
     int dense_m;   // unknowns of the coarsest level
     int singular;
@@ -939,17 +940,23 @@ struct BulkLoad {
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
     }
 };
-// every thread waits for the copies: a microsecond or so, with a limit (on giving up the values are
-// wrong, the residual does not fall and the solve reports it)
-__device__ __forceinline__ void bulk_wait(unsigned long long* b) {
+// Waits for the copies, a microsecond or so: every thread of the block calls it, and all get the same
+// answer. False after BULK_WAIT cycles (about a second): the data is not there and may still be on
+// its way. The kernel then sets MG_WAIT_RAN_OUT, which ends the solve and reaches the host
+// (CPIC_ERR_TIMEOUT), and waits once more before it leaves, as the copies write its memory.
+constexpr long long BULK_WAIT = 1ll << 31;
+__device__ __forceinline__ bool bulk_wait(unsigned long long* b) {
     const unsigned bar = (unsigned)__cvta_generic_to_shared(b);
+    const long long start = clock64();
     unsigned done = 0;
-    for (int spin = 0; spin < (1 << 20) && !done; ++spin)
+    do {
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(done)
             : "r"(bar)
             : "memory");
+    } while (!done && clock64() - start < BULK_WAIT);
+    return !__syncthreads_or(!done);
 }
 
 // Lays the one-CTA levels out in shared memory from word off on (per smoothed level A [NPT], dinv,
@@ -1088,8 +1095,11 @@ __global__ void __launch_bounds__(512, 1) coarse_cycle_kernel(const __grid_const
         T[S.first_cta].x[c] = 0.0f;
         if (!smoothed) T[S.first_cta].b[c] = G.b[c];
     }
-    bulk_wait(&bar);
-    __syncthreads();
+    if (!bulk_wait(&bar)) {
+        if (tid == 0) *S.status = MG_WAIT_RAN_OUT;
+        (void)bulk_wait(&bar);
+        return;
+    }
     cta_cycle<D, NPT>(S, V, T, dense_smem ? sm + dense_smem : nullptr, nu1, nu2);
     for (int c = tid; c < G.ncell; c += nt) G.x[c] = T[S.first_cta].x[c];
 }
@@ -1197,7 +1207,9 @@ __global__ void __launch_bounds__(512, 1) coarse_cluster_kernel(const __grid_con
     for (int t = 0; t < P.ns; ++t)
         for (int c = tid; c < (W[t].R + 2) * W[t].plane; c += 512) W[t].x[c] = 0.0f;
     for (int c = tid; c < T[S.first_cta].ncell; c += 512) T[S.first_cta].x[c] = 0.0f;
-    bulk_wait(&bar);
+    const bool loaded = bulk_wait(&bar);
+    // (a CTA whose wait ran out keeps to the barriers, on values that nobody uses)
+    if (!loaded && tid == 0) *S.status = MG_WAIT_RAN_OUT;
     cl.sync();  // every CTA's x is set before a neighbour writes into it
     for (int t = 0; t < P.ns; ++t) {
         const Slab L = W[t];
@@ -1303,6 +1315,7 @@ __global__ void __launch_bounds__(512, 1) coarse_cluster_kernel(const __grid_con
     const Slab L = W[0];
     float* out = S.l[P.first].x + L.z0 * L.plane;
     for (int c = tid; c < L.R * L.plane; c += 512) out[c] = L.x[L.plane + c];
+    if (!loaded) (void)bulk_wait(&bar);
 }
 
 // ------------------------------------------------------------------ FP64 outer iteration
@@ -1443,8 +1456,9 @@ __global__ void __launch_bounds__(256) residual_kernel(const __grid_constant__ R
         double res = bnorm > 0.0 ? sqrt(a) / bnorm : 0.0;
         ctr->mg_residual = res;
         bool converged = res <= P.rtol;
-        if (converged) ctr->mg_converged = 1;
-        bool cont = !converged && ctr->mg_cycles < P.max_cycles;
+        const bool lost = ctr->mg_converged == MG_WAIT_RAN_OUT;  // a V-cycle's data did not arrive
+        if (converged) set_converged(ctr);
+        bool cont = !converged && !lost && ctr->mg_cycles < P.max_cycles;
         *P.done = cont ? 0 : 1;
         if (P.use_handle) cudaGraphSetConditional(P.handle, cont ? 1u : 0u);
     }
@@ -1686,8 +1700,11 @@ __global__ void __launch_bounds__(CS_THREADS, 1) cta_solve_kernel(const __grid_c
     }
     __syncthreads();  // the barrier is initialised before any other thread waits on it
     for (int c = tid; c < n; c += CS_THREADS) phi[c] = P.phi[c];
-    bulk_wait(&bar);
-    __syncthreads();
+    if (!bulk_wait(&bar)) {
+        if (tid == 0) *S.status = MG_WAIT_RAN_OUT;
+        (void)bulk_wait(&bar);
+        return;
+    }
     const CtaLevel L = T[0];
     const float* dense = P.odense ? sm + P.odense : nullptr;
     auto steps = [&](int c) {
@@ -1731,7 +1748,7 @@ __global__ void __launch_bounds__(CS_THREADS, 1) cta_solve_kernel(const __grid_c
             P.ctr->mg_cycles = cycles;
             P.ctr->mg_residual = res;
             P.ctr->mg_bnorm = bnorm;
-            if (res <= P.rtol) P.ctr->mg_converged = 1;
+            if (res <= P.rtol) set_converged(P.ctr);
         }
         if (res <= P.rtol || cycles >= P.max_cycles) break;
         // p, and the V-cycle on it
@@ -2096,6 +2113,7 @@ LVSet make_set(const cpic_run* r) {
     S.nl = r->nlevels;
     S.line = r->mg_smoother == CPIC_MG_SMOOTH_LINE ? 1 : 0;
     for (int l = 0; l < r->nlevels; ++l) S.l[l] = make_lv<float>(r, l, true);
+    S.status = &r->ctr->mg_converged;
     S.dense_inv = r->dense_inv32;
     S.dense_m = (int)r->lev[r->nlevels - 1].ncell;
     S.singular = r->singular ? 1 : 0;
@@ -2655,6 +2673,7 @@ int mg_solve(cpic_run* r, double rtol, int max_cycles, bool fold, int* cycles, d
         CPIC_CUDA(cudaStreamSynchronize(r->stream));
         if (cycles) *cycles = h.mg_cycles;
         if (res) *res = h.mg_residual;
+        if (h.mg_converged == MG_WAIT_RAN_OUT) return wait_ran_out();
         if (!h.mg_converged) {
             set_error("multigrid: relative residual %.3e > %.3e after %d cycles", h.mg_residual, rtol, h.mg_cycles);
             return CPIC_ERR_NOT_CONVERGED;

@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) mg_cluster_kernel(const __grid_
         P.ctr->mg_cycles = cycles;
         P.ctr->mg_residual = res;
         P.ctr->mg_bnorm = sqrt(bb);
-        if (s_next == 0) P.ctr->mg_converged = 1;
+        if (s_next == 0) set_converged(P.ctr);
     }
     cl.sync();  // no CTA leaves while another may still write to its shared memory
 }

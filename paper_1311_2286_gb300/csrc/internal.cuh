@@ -71,6 +71,11 @@ struct DevCounters {
     int perm;
 };
 
+// The stopping test of every form of the solve is relative_residual <= rtol: met at once when b is
+// zero, never by a residual or a b that is not a number or infinite.
+__device__ __forceinline__ double relative_residual(double rr, double bnorm) {
+    return bnorm == 0.0 ? 0.0 : sqrt(rr) / bnorm;
+}
 __device__ __forceinline__ void set_converged(DevCounters* ctr) {
     if (ctr->mg_converged != MG_WAIT_RAN_OUT) ctr->mg_converged = 1;
 }

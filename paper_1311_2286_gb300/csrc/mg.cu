@@ -1452,8 +1452,7 @@ __global__ void __launch_bounds__(256) residual_kernel(const __grid_constant__ R
                 ks->rho = h;
             }
         }
-        const double bnorm = ctr->mg_bnorm;
-        double res = bnorm > 0.0 ? sqrt(a) / bnorm : 0.0;
+        const double res = relative_residual(a, ctr->mg_bnorm);
         ctr->mg_residual = res;
         bool converged = res <= P.rtol;
         const bool lost = ctr->mg_converged == MG_WAIT_RAN_OUT;  // a V-cycle's data did not arrive
@@ -1743,7 +1742,7 @@ __global__ void __launch_bounds__(CS_THREADS, 1) cta_solve_kernel(const __grid_c
     rho = sum[0];
     int cycles = 0;
     for (;;) {
-        const double res = bnorm > 0.0 ? sqrt(sum[0]) / bnorm : 0.0;
+        const double res = relative_residual(sum[0], bnorm);
         if (tid == 0) {
             P.ctr->mg_cycles = cycles;
             P.ctr->mg_residual = res;

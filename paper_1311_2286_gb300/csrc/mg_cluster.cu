@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) mg_cluster_kernel(const __grid_
     const int tid = threadIdx.x;
     __shared__ double red64[CL_THREADS];
     __shared__ float redf[CL_THREADS / 32];
-    __shared__ double s_bb, s_rr;
+    __shared__ double s_bn, s_res;  // ||b||, ||r|| / ||b||
     __shared__ float s_scale;  // 1 / ||b||
     __shared__ int s_next;  // 0: within the tolerance, 1: cycle, residual in FP64, 2: cycle, in pairs
     const ClLevel L0 = P.L[0];
@@ -366,16 +366,17 @@ __global__ void __launch_bounds__(CL_THREADS, 1) mg_cluster_kernel(const __grid_
                 }
                 if (tid == 0) {
                     if (start) {
-                        s_bb = b;
-                        s_scale = (float)(1.0 / sqrt(b));
+                        s_bn = sqrt(b);
+                        s_scale = (float)(1.0 / s_bn);
                     }
-                    s_rr = a;
-                    s_next = !(a > P.rtol * P.rtol * s_bb) ? 0 : (a < (double)(DF_FROM * DF_FROM) * s_bb ? 2 : 1);
+                    s_res = relative_residual(a, s_bn);
+                    s_next = s_res <= P.rtol ? 0 : (s_res < (double)DF_FROM ? 2 : 1);
                 }
             } else {
                 float a = tid < cs ? partf[16 * q + tid] : 0.0f;
 #pragma unroll
                 for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                // (one that is not a number goes to the FP64 residual, which decides)
                 if (tid == 0) s_next = !(a > P.rtol2) ? 0 : (a < DF_FROM * DF_FROM ? 2 : 1);
             }
         }
@@ -586,10 +587,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) mg_cluster_kernel(const __grid_
         exact = to64;
     }
     if (rank == 0 && tid == 0) {
-        const double bb = s_bb, res = bb > 0.0 ? sqrt(s_rr) / sqrt(bb) : 0.0;
         P.ctr->mg_cycles = cycles;
-        P.ctr->mg_residual = res;
-        P.ctr->mg_bnorm = sqrt(bb);
+        P.ctr->mg_residual = s_res;
+        P.ctr->mg_bnorm = s_bn;
         if (s_next == 0) set_converged(P.ctr);
     }
     cl.sync();  // no CTA leaves while another may still write to its shared memory

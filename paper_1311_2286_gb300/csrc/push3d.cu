@@ -575,9 +575,12 @@ __global__ void __launch_bounds__(P3_THREADS, 3) push3d_kernel(PushParams p) {
 // per-warp transposition: every lane writes its 27 node weights (spec Q) into its row of the
 // warp's shared buffer; then lane j (j < 27) sums node j over the rows of each run of
 // consecutive lanes that came from one cell (particles are kept in cell order, so a warp has
-// one to three runs) and adds the run's sum with one 64-bit atomic. Particles that left
-// their cell are taken out of their run's sum and added at their own cell: runs of equal new
-// cells instead are cut by every such particle, twice (half the lanes' worth of 27-lane
+// one to three runs) and adds the run's sum with one 64-bit atomic. (A warp of more than
+// MANY_RUNS, out of order or at a few particles a cell, walks its 32 rows once and cuts them where
+// the new cell changes: a loop per run is a chain of short loads. Eight steps from a sort on, 64^3
+// cells: 1 M particles 658 us, 742 without that; 8 M 4430 and 4680 us; sorted at every step the same.)
+// Particles that left their cell are taken out of their run's sum and added at their own cell: runs of
+// equal new cells instead are cut by every such particle, twice (half the lanes' worth of 27-lane
 // atomics for electrons, a third of them move a cell per step). The order of integer additions
 // does not change the result. No deposit tile: the kernel needs 28 KB of shared memory per
 // block. Three blocks per SM at 80 registers: at 64 it spills (64M particles with the sort's
@@ -586,6 +589,7 @@ __global__ void __launch_bounds__(P3_THREADS, 3) push3d_kernel(PushParams p) {
 // and movers 1160.
 constexpr int PD_THREADS = 256;
 constexpr int PD_STRIDE = 28;  // words per lane row: 27 node weights and one zero
+constexpr int MANY_RUNS = 4;   // (2 to 8 measured alike, 12 and more slower)
 
 // old: padded offset of the cell the slot's particle came from (-1: empty slot); hist: the next
 // sort's counts of the species, or null; the particle's number among its new cell's goes to *rank
@@ -617,8 +621,10 @@ __device__ __forceinline__ void deposit_runs3(const PushParams& p, int s, bool a
     }
     row[13] = (alive ? 1u << QF : 0u) - rest;
     const int off = alive ? c[0] + c[1] * p.hs1 + c[2] * p.hs2 : -1;
-    const int next = __shfl_down_sync(FULL, old, 1);  // every lane takes part (lane 31 gets its own)
+    // every lane takes part (lane 31 gets its own)
+    const int next = __shfl_down_sync(FULL, old, 1), next_off = __shfl_down_sync(FULL, off, 1);
     unsigned ends = __ballot_sync(FULL, lane == 31 || next != old);
+    const unsigned ends_off = __ballot_sync(FULL, lane == 31 || next_off != off);
     const unsigned stay = __ballot_sync(FULL, alive && off == old);
     const unsigned move = __ballot_sync(FULL, alive && off != old);
     int number = 0, first = lane;  // the atomic's value, held by lane `first`
@@ -658,6 +664,17 @@ __device__ __forceinline__ void deposit_runs3(const PushParams& p, int s, bool a
 #pragma unroll
         for (int r = 0; r < 32; ++r) acc[r & 3] += col[r * PD_STRIDE];
         finish((acc[0] + acc[1]) + (acc[2] + acc[3]), FULL, 31);
+    } else if (__popc(ends) > MANY_RUNS) {
+        unsigned acc = 0;
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+            acc += col[r * PD_STRIDE];
+            if ((ends_off >> r) & 1u) {  // warp-uniform
+                const int o = __shfl_sync(FULL, off, r);
+                if (o >= 0 && lane < 27) atomicAdd(g + o, (unsigned long long)acc);
+                acc = 0;
+            }
+        }
     } else {
         int a = 0;
         for (; ends; ends &= ends - 1u) {

@@ -88,7 +88,9 @@ __device__ __forceinline__ void tile_add_row(unsigned& m, unsigned a, unsigned q
 // Deposit of one particle per lane into the chunk's tile; lanes whose 3x3 stencil leaves the
 // tile rows deposit straight into the padded global grid. Lanes that share a cell are summed
 // first (__reduce_add_sync over each such group) and deposited by one lane of the group.
-// peers: the lanes of this lane's new cell (alive lanes; the others hold keys of their own).
+// With MATCHED, peers holds the lanes of this lane's new cell (alive lanes; the others hold keys of
+// their own); else they are looked for here.
+template <bool MATCHED>
 __device__ __forceinline__ void deposit_tile(const PushParams& p, const Tile& tl, int s, bool alive,
                                              const int* c, const float* t, unsigned peers) {
     const int lane = threadIdx.x & 31;
@@ -102,6 +104,7 @@ __device__ __forceinline__ void deposit_tile(const PushParams& p, const Tile& tl
     // every group of lanes that share a cell (all of them in the tile or none) is summed over its
     // lanes and deposited by its lowest lane
     const int off = rr * tl.W + c[0] + 1;
+    if (!MATCHED) peers = __match_any_sync(FULL, in ? off : -1 - lane);
     const int my_leader = __ffs(peers) - 1;
     const bool issue = in && lane == my_leader;
     for (unsigned g = __ballot_sync(FULL, issue && (peers & (peers - 1u)) != 0u); g; g &= g - 1u) {
@@ -244,9 +247,11 @@ __device__ __forceinline__ void push2d_run(const PushParams& p, int bid, int nb,
             nv1_ = vp[T + j];
             nv2_ = vp[2 * T + j];
         }
-        // the iteration loop, specialised on whether the chunk's tile is in use
-        auto iterate = [&](auto tile_tag) {
-            constexpr bool TILE = decltype(tile_tag)::value;
+        // the iteration loop, specialised on whether the chunk's tile is in use and whether the
+        // step counts for the sort (a step that does not has no use for the lanes of a cell before
+        // the deposit: the match costs 512 x 1024 cells' push 6 %)
+        auto iterate = [&](auto tile_tag, auto count_tag) {
+            constexpr bool TILE = decltype(tile_tag)::value, COUNT = decltype(count_tag)::value;
             for (int base = lo; base < hi; base += P2_THREADS) {
                 const int slot = i;
                 const int cw = ncw;
@@ -384,28 +389,34 @@ __device__ __forceinline__ void push2d_run(const PushParams& p, int bid, int nb,
                 // spec D: v_old . v_new as an FP32 fma chain, then round(x 2^24) to int64
                 const float ke32 = __fmaf_rn(vo2, v[2], __fmaf_rn(vo1, v[1], __fmul_rn(vo0, v[0])));
                 if (active) ke += __float2ll_rn(__fmul_rn(ke32, 16777216.0f));
-                const int lane = threadIdx.x & 31, key = alive ? cn[0] + n0 * cn[1] : -1 - lane;
-                const unsigned peers = __match_any_sync(FULL, key);
+                const int lane = threadIdx.x & 31;
+                unsigned peers = 0u;
                 int number = 0;
-                if (p.hist && alive && __ffs(peers) - 1 == lane)  // the next sort's counts
-                    number = atomicAdd(p.hist + (size_t)s * n0 * n1 + key, (int)__popc(peers));
+                if constexpr (COUNT) {  // the next sort's counts
+                    const int key = alive ? cn[0] + n0 * cn[1] : -1 - lane;
+                    peers = __match_any_sync(FULL, key);
+                    if (alive && __ffs(peers) - 1 == lane)
+                        number = atomicAdd(p.hist + (size_t)s * n0 * n1 + key, (int)__popc(peers));
+                }
                 store_state(active, cellq + slot, alive ? (cn[0] | (cn[1] << 16)) : -1, tq + slot, tn[0],
                             tq + T + slot, tn[1], vq + slot, v[0], vq + T + slot, v[1], vq + 2 * T + slot, v[2]);
                 // a6: deposit
                 if constexpr (TILE)
-                    deposit_tile(p, tl, s, alive, cn, tn, peers);
+                    deposit_tile<COUNT>(p, tl, s, alive, cn, tn, peers);
                 else
                     deposit_warp<2>(p, s, alive, cn, tn);
-                if (p.hist) {  // the particle's number among its cell's, once the atomic is back
+                if constexpr (COUNT) {  // the particle's number among its cell's, once the atomic is back
                     number = __shfl_sync(FULL, number, __ffs(peers) - 1);
                     if (alive) p.rank[b0 + slot] = number + __popc(peers & ((1u << lane) - 1u));
                 }
             }
         };
-        if (tl.on)
-            iterate(std::true_type{});
-        else
-            iterate(std::false_type{});
+        auto counted = [&](auto tile_tag) {
+            if (p.hist) iterate(tile_tag, std::true_type{});
+            else iterate(tile_tag, std::false_type{});
+        };
+        if (tl.on) counted(std::true_type{});
+        else counted(std::false_type{});
         // flush the tile into the padded grid (rows -1 .. n1 exist there; the others hold
         // nothing)
         if (tl.on) {

@@ -623,6 +623,11 @@ void invalidate_graphs(cpic_run* r) {
         }
 }
 
+void set_sort_interval(cpic_run* r, int interval) {
+    if (push_window(interval) != push_window(r->cfg.sort_interval)) invalidate_graphs(r);
+    r->cfg.sort_interval = interval;
+}
+
 namespace {
 
 cudaEvent_t pool_event(cpic_run* r) {
@@ -864,7 +869,7 @@ int cpic_set_sort_interval(cpic_run* r, int interval) {
         set_error("set_sort_interval: NULL run or negative interval");
         return CPIC_ERR_INVALID;
     }
-    r->cfg.sort_interval = interval;
+    set_sort_interval(r, interval);
     return CPIC_OK;
 }
 

@@ -131,6 +131,7 @@ struct PushParams {
     float gb[3];                   // its unit field direction b (velocity components' basis)
     float gy[CPIC_MAX_SPECIES][4]; // per species cos th, sin th, sin th / th, (1 - cos th) / th
     int chunk;                     // particles per block chunk (0: one wave of blocks)
+    int window;                    // sorted every few steps (see push_window)
     int* hist;                     // when set: count each kept particle's new cell here
                                    // ([species][cell], the next sort's histogram), and leave
     int* rank;                     // the particle's number among its cell's per slot here
@@ -293,6 +294,9 @@ int launch_push_kernel(cpic_run* r);  // the fused push + deposit kernel alone
 // whether that kernel also ends the push (else launch_finalize_step follows it)
 bool push_finalizes(const cpic_run* r);
 PushParams make_push_params(cpic_run* r);
+// whether the 2D push works through the particles in small chunks: sorted at least every eighth step
+inline bool push_window(int sort_interval) { return sort_interval > 0 && sort_interval <= 8; }
+void set_sort_interval(cpic_run* r, int interval);  // captured steps hold push_window
 void set_boris_constants(const cpic_run* r, PushParams* p, double fraction);
 int launch_push2d(cpic_run* r, const PushParams& p);
 // batched 2D particle step (row a11): one launch over a device table of runs' parameters

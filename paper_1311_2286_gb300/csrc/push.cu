@@ -416,6 +416,7 @@ PushParams make_push_params(cpic_run* r) {
     p.origin = 1 + p.hs1 + p.hs2;
     p.ctr = r->ctr;
     p.chunk = r->push_chunk;
+    p.window = push_window(r->cfg.sort_interval);
     p.hist = r->count_hist ? r->hist : nullptr;
     p.rank = r->prank;
     p.tile = r->push_tile;

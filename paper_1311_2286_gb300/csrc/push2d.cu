@@ -162,12 +162,16 @@ __device__ __forceinline__ void push2d_run(const PushParams& p, int bid, int nb,
         total += cnt[s];
     }
     if (total == 0) return;
-    // chunk size: a multiple of the block. Unless set, a block's share is cut into equal chunks of at most AUTO_CHUNK particles: the blocks
-    // then work in a window that advances through the particles, and what a push reads through a
-    // pending order across chunks (a particle that moved a row) is still in L2 when its own
-    // chunk comes (64M particles on 512 x 1024: one chunk a block 1672 us, 8192: 1452 us, 1024: 1749)
+    // chunk size: a multiple of the block. Unless set, a block's share, cut into equal chunks of at most
+    // AUTO_CHUNK particles where the particles are sorted every few steps (p.window): the blocks then
+    // work in a window that advances through the particles, and what a push reads through a pending
+    // order across chunks (a particle that moved a row) is still in L2 when its own chunk comes (64M
+    // particles on 512 x 1024: one chunk a block 1672 us, 8192: 1452 us, 1024: 1749; 16M sorted every
+    // fourth step: four steps 1760 and 1660 us). Long after a sort the small chunks cost more than
+    // they save: their rows no longer fit the tile, or are other blocks' too (8M particles on 64 x 64
+    // cells, the 40 steps from a sort on: 9863 us, one chunk a block 9100).
     constexpr int AUTO_CHUNK = 8192;
-    const int share = (total + nb - 1) / nb, cuts = (share + AUTO_CHUNK - 1) / AUTO_CHUNK;
+    const int share = (total + nb - 1) / nb, cuts = p.window ? (share + AUTO_CHUNK - 1) / AUTO_CHUNK : 1;
     const int C = p.chunk > 0 ? p.chunk : ((share + cuts - 1) / cuts + P2_THREADS - 1) / P2_THREADS * P2_THREADS;
     const int n0 = p.n[0], n1 = p.n[1], nv0 = n0 + 1;
     const float4* __restrict__ K4 = reinterpret_cast<const float4*>(p.K);

@@ -129,7 +129,7 @@ int cpic_autotune(cpic_run* r, int trial_steps, cpic_tuning* out) {
     int best = saved_interval > 0 ? saved_interval : 4;
     float best_ms = 0.0f;
     for (int c = 0; !st && c < CPIC_TUNE_CANDIDATES; ++c) {
-        r->cfg.sort_interval = intervals[c];
+        set_sort_interval(r, intervals[c]);
         out->interval[c] = intervals[c];
         st = tune_trial(r, buf, saved_cur, trial_steps, a, b, &out->ms_per_step[c]);
         if (!st && (best_ms == 0.0f || out->ms_per_step[c] < best_ms)) {
@@ -137,7 +137,7 @@ int cpic_autotune(cpic_run* r, int trial_steps, cpic_tuning* out) {
             best = intervals[c];
         }
     }
-    r->cfg.sort_interval = st ? saved_interval : best;
+    set_sort_interval(r, st ? saved_interval : best);
     // 2. particles per block chunk, at that interval
     int best_chunk = saved_chunk;
     best_ms = 0.0f;
@@ -168,18 +168,18 @@ int cpic_autotune(cpic_run* r, int trial_steps, cpic_tuning* out) {
         best = r->cfg.sort_interval;
         best_ms = 0.0f;
         for (int c = 0; !st && c < CPIC_TUNE_CANDIDATES; ++c) {
-            r->cfg.sort_interval = intervals[c];
+            set_sort_interval(r, intervals[c]);
             st = tune_trial(r, buf, saved_cur, trial_steps, a, b, &out->ms_per_step[c]);
             if (!st && (best_ms == 0.0f || out->ms_per_step[c] < best_ms)) {
                 best_ms = out->ms_per_step[c];
                 best = intervals[c];
             }
         }
-        r->cfg.sort_interval = best;
+        set_sort_interval(r, best);
     }
     r->steps_since_sort = saved_since;
     if (st) {
-        r->cfg.sort_interval = saved_interval;
+        set_sort_interval(r, saved_interval);
         cpic_set_push_tuning(r, saved_chunk, saved_tile);
     }
     out->sort_interval = r->cfg.sort_interval;

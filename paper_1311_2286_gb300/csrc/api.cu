@@ -1002,6 +1002,9 @@ int cpic_destroy(cpic_run* r) {
     for (cudaEvent_t ev : *r->prof_pool) cudaEventDestroy(ev);
     invalidate_graphs(r);
     if (r->capture_stream) cudaStreamDestroy(r->capture_stream);
+    if (r->done_host) cudaFreeHost(r->done_host);
+    for (cudaEvent_t ev : r->done_event)
+        if (ev) cudaEventDestroy(ev);
     delete r->prof_events;
     delete r->prof_pool;
     delete r;

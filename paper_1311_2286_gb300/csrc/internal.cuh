@@ -219,6 +219,8 @@ struct cpic_run {
     int graph_kernels[2][2];           // kernel nodes launched by one replay
     bool graph_sort_fused[2][2];       // the graph's sort leaves its order to the next push
     cudaStream_t capture_stream;
+    int* done_host;              // page-locked: the done flags of the last two cycles (mg_solve), and
+    cudaEvent_t done_event[2];   // the events after them; created when first needed
     int cluster_cs;              // cluster size of the cluster solver (0: not applicable)
     int cluster_nd;              // its split levels
     bool cluster_class;          // V-cycles are the outer iteration, also where no cluster layout fits

@@ -92,3 +92,19 @@ def test_nothing_to_solve_ends_at_once(cpic, form):
     d = run.diag()
     assert d["mg_cycles"] == 0 and d["mg_residual"] == 0.0
     assert np.array_equal(run.phi(), phi)
+
+
+# (the cluster kernel ends its own loop, and takes the residual of its last permitted cycle in FP64)
+@pytest.mark.parametrize("form", [f for f in FORMS if f != "cluster"], indirect=True)
+def test_a_cycle_enqueued_beyond_the_last_leaves_the_potential(cpic, form):
+    """The cycle that a host one ahead has enqueued when the solve ends changes nothing: the potential
+    is that of a solve cut off at the same number of cycles, and solving again does none."""
+    run, phi = form(-5.0)
+    run.set_phi(phi)
+    cycles, res = run.solve_field(rtol=1e-9, max_cycles=100)
+    first = run.phi()
+    run.set_phi(phi)
+    assert run.solve_field(rtol=1e-9, max_cycles=cycles) == (cycles, res)
+    assert np.array_equal(run.phi(), first)
+    assert run.solve_field(rtol=1e-9, max_cycles=100) == (0, res)
+    assert np.array_equal(run.phi(), first)

@@ -141,12 +141,15 @@ int64_t cpic_kernel_launches(void);
 /* ---------------------------------------------------------------- setup */
 
 /* Device bytes a run with this configuration needs (the size of a caller arena).
- * Pure host computation; no GPU work. */
+ * Pure host computation; no GPU work. With a sort interval it includes 4 bytes a particle slot
+ * for the numbers that make a step's sort cheap (2D runs without reflecting boundaries that are
+ * not axisymmetric, and 3D runs of the shell's and of wholly periodic boundaries). */
 int cpic_query_footprint(const cpic_config* cfg, size_t* device_bytes);
 
 /* Create a run on the current device. arena: NULL (the run cudaMallocs its memory) or a
  * device buffer of at least cpic_query_footprint bytes, 256-byte aligned, owned by the
- * caller. stream: cudaStream_t to enqueue on (NULL = legacy default stream). */
+ * caller (one that is short of the sort's numbers only is taken, as is a device whose memory is:
+ * the run then sorts without them). stream: cudaStream_t to enqueue on (NULL = legacy default stream). */
 int cpic_create(const cpic_config* cfg, void* arena, size_t arena_bytes, void* stream,
                 cpic_run** out);
 /* The run's configuration as in use (the sort interval as last chosen by cpic_autotune). */

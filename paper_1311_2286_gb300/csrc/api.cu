@@ -169,6 +169,17 @@ int plan_levels(const cpic_config* c, int lev_n[MAX_LEVELS][3], int* nl) {
     return CPIC_OK;
 }
 
+// Whether a run is given room for its particles' numbers (4 bytes a slot; with them a sort is a third
+// of what it is without, see place_kernel): when it sorts, by a push that can number (see
+// push_fused_ok; a magnetic field set later leaves the room unused).
+bool numbers_particles(const cpic_config& c) {
+    if (c.sort_interval <= 0 || c.axisymmetric) return false;
+    if (c.dim == 3) return push3d_special(c);
+    for (int f = 0; f < 4; ++f)
+        if (c.particle_bc[f] == CPIC_PBC_REFLECT) return false;
+    return true;
+}
+
 void plan(cpic_run* r, Planner& P) {
     const cpic_config& c = r->cfg;
     int D = r->D;
@@ -228,7 +239,7 @@ void plan(cpic_run* r, Planner& P) {
     r->kv = P.take<double>((size_t)2 * r->ncell + ((size_t)3 * r->ncell + 1) / 2);  // r, r^; FP32 p, v, s
     r->ph32 = P.take<float>(r->ncell);
     r->hist = P.take<int>((size_t)c.n_species * r->ncell);
-    r->prank = P.take<int>(total);
+    r->prank = r->numbered ? P.take<int>(total) : nullptr;
     r->scan = P.take<long long>((size_t)c.n_species * r->ncell + 1);
     r->scan_blocks = P.take<long long>(1025);
     for (int l = 0; l < r->nlevels; ++l) {
@@ -849,6 +860,7 @@ int cpic_query_footprint(const cpic_config* cfg, size_t* bytes) {
     init_geometry_sizes(&tmp, cfg);
     st = setup_levels(&tmp);
     if (st) return st;
+    tmp.numbered = numbers_particles(*cfg);
     Planner P;
     plan(&tmp, P);
     *bytes = P.used + 256;
@@ -943,9 +955,15 @@ int cpic_create(const cpic_config* cfg, void* arena, size_t arena_bytes, void* s
         return st;
     }
     r->stream = (cudaStream_t)stream;
-    Planner dry;
-    plan(r, dry);
-    size_t need = dry.used + 256;
+    auto planned = [&](bool numbered) {
+        r->numbered = numbered;
+        Planner dry;
+        plan(r, dry);
+        return dry.used + 256;
+    };
+    size_t need = planned(numbers_particles(*cfg));
+    // the numbers are left out where only they do not fit
+    if (arena && arena_bytes < need && r->numbered) need = planned(false);
     if (arena) {
         if (arena_bytes < need || (reinterpret_cast<uintptr_t>(arena) & 255)) {
             set_error("arena too small or misaligned: need %zu bytes, 256-byte aligned", need);
@@ -957,6 +975,11 @@ int cpic_create(const cpic_config* cfg, void* arena, size_t arena_bytes, void* s
     } else {
         void* p = nullptr;
         cudaError_t e = cudaMalloc(&p, need);
+        if (e == cudaErrorMemoryAllocation && r->numbered) {
+            (void)cudaGetLastError();
+            need = planned(false);
+            e = cudaMalloc(&p, need);
+        }
         if (e != cudaSuccess) {
             set_error("cudaMalloc(%zu) failed: %s", need, cudaGetErrorString(e));
             delete r;

@@ -277,8 +277,10 @@ __global__ void inject_kernel(InjectParams ip) {
             }
             long long slot = p.pb.base[s] + start + pi;
             p.pb.cell[cur][slot] = alive ? encode<2>(c) : -1;
-            if (p.hist && alive)  // the push numbers each cell's particles for the sort: the newcomers too
-                p.rank[slot] = atomicAdd(p.hist + (size_t)s * n1 * n2 + c[0] + (size_t)n1 * c[1], 1);
+            if (p.hist && alive) {  // the push numbers each cell's particles for the sort: the newcomers too
+                const int number = atomicAdd(p.hist + (size_t)s * n1 * n2 + c[0] + (size_t)n1 * c[1], 1);
+                if (p.rank) p.rank[slot] = number;
+            }
             p.pb.t[cur][slot] = tt[0];
             p.pb.t[cur][T + slot] = tt[1];
             p.pb.v[cur][slot] = v0;
@@ -392,9 +394,11 @@ __global__ void inject3d_kernel(InjectParams ip) {
             alive = c[0] >= 0 && c[0] < n1 && c[1] >= 0 && c[1] < n2;
             const long long slot = p.pb.base[s] + start + pi;
             p.pb.cell[cur][slot] = alive ? encode<3>(c) : -1;
-            if (p.hist && alive)  // the push numbers each cell's particles for the sort: the newcomers too
-                p.rank[slot] =
+            if (p.hist && alive) {  // the push numbers each cell's particles for the sort: the newcomers too
+                const int number =
                     atomicAdd(p.hist + (size_t)s * n1 * n2 * n3 + c[0] + (size_t)n1 * (c[1] + (size_t)n2 * c[2]), 1);
+                if (p.rank) p.rank[slot] = number;
+            }
 #pragma unroll
             for (int a = 0; a < 3; ++a) p.pb.t[cur][a * T + slot] = tt[a];
 #pragma unroll

@@ -134,7 +134,7 @@ struct PushParams {
     int window;                    // sorted every few steps (see push_window)
     int* hist;                     // when set: count each kept particle's new cell here
                                    // ([species][cell], the next sort's histogram), and leave
-    int* rank;                     // the particle's number among its cell's per slot here
+    int* rank;                     // the particle's number among its cell's per slot here, if not null
     int tile;                      // 1: shared-memory deposit tile when the chunk fits
     unsigned* fin;                 // when set: block counter, the last block to finish ends the
                                    // step's push (step count, buffer flip of a pending order)
@@ -226,8 +226,8 @@ struct cpic_run {
     bool cluster_class;          // V-cycles are the outer iteration, also where no cluster layout fits
     int slab_cs;                 // largest cluster of the 3D V-cycle's cluster part (0: none)
     bool order_pending;          // a fused sort's order may be pending on the device (DevCounters::perm)
-    bool count_hist;             // this step's push and injection count the cells (hist) and number
-                                 // the particles in them (prank)
+    bool count_hist;             // this step's push and injection count the cells (hist) and, with
+                                 // room for it, number the particles in them (prank)
     int dense_m;                 // coarsest unknowns (+1 row when singular)
     bool singular;
     double sumJ;                 // sum of finest J_c (singular projection)
@@ -255,7 +255,8 @@ struct cpic_run {
     float* ph32;                 // preconditioned direction p_hat (FP32)
     // sort scratch
     int* hist;                   // [nsp][ncell] counts (-> cursors of the rank pass)
-    int* prank;                  // [slot] a particle's number among its cell's (counted steps)
+    bool numbered;               // there is room for prank (see numbers_particles)
+    int* prank;                  // [slot] a particle's number among its cell's (counted steps), or null
     long long* scan;             // [nsp*ncell + 1] exclusive prefix
     long long* scan_blocks;      // block partials
     // injection
@@ -328,6 +329,7 @@ int launch_sort(cpic_run* r, bool fused = false);
 int resolve_order(cpic_run* r);
 bool push_fused_ok(const cpic_run* r);
 bool push3d_direct_taken(const cpic_run* r);
+bool push3d_special(const cpic_config& c);  // the axis kinds push3d.cu is instantiated for
 // mg.cu
 int mg_setup(cpic_run* r);
 // fold: the charge is still in the padded deposit grid

@@ -526,11 +526,7 @@ bool push_fused_ok(const cpic_run* r) {
 
 bool push_finalizes(const cpic_run* r) {
     if (r->magnetized) return false;
-    if (r->D == 3) {
-        const int k0 = r->cfg.particle_bc[0], k1 = r->cfg.particle_bc[2], k2 = r->cfg.particle_bc[4];
-        return (k0 == CPIC_PBC_ABSORB && k1 == CPIC_PBC_REFLECT && k2 == CPIC_PBC_PERIODIC) ||
-               (k0 == CPIC_PBC_PERIODIC && k1 == CPIC_PBC_PERIODIC && k2 == CPIC_PBC_PERIODIC);
-    }
+    if (r->D == 3) return push3d_special(r->cfg);
     return !r->cfg.axisymmetric && r->cfg.particle_bc[0] != CPIC_PBC_REFLECT && r->cfg.particle_bc[1] != CPIC_PBC_REFLECT &&
            r->cfg.particle_bc[2] != CPIC_PBC_REFLECT && r->cfg.particle_bc[3] != CPIC_PBC_REFLECT;
 }

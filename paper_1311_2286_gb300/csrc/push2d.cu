@@ -409,7 +409,7 @@ __device__ __forceinline__ void push2d_run(const PushParams& p, int bid, int nb,
                     deposit_tile<COUNT>(p, tl, s, alive, cn, tn, peers);
                 else
                     deposit_warp<2>(p, s, alive, cn, tn);
-                if constexpr (COUNT) {  // the particle's number among its cell's, once the atomic is back
+                if (COUNT && p.rank) {  // the particle's number among its cell's, once the atomic is back
                     number = __shfl_sync(FULL, number, __ffs(peers) - 1);
                     if (alive) p.rank[b0 + slot] = number + __popc(peers & ((1u << lane) - 1u));
                 }

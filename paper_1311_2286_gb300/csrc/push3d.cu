@@ -592,8 +592,8 @@ constexpr int PD_STRIDE = 28;  // words per lane row: 27 node weights and one ze
 constexpr int MANY_RUNS = 4;   // (2 to 8 measured alike, 12 and more slower)
 
 // old: padded offset of the cell the slot's particle came from (-1: empty slot); hist: the next
-// sort's counts of the species, or null; the particle's number among its new cell's goes to *rank
-// (the count's atomic returns it; it is stored last, so that its latency overlaps the deposit)
+// sort's counts of the species, or null; the particle's number among its new cell's goes to *rank,
+// unless that is null (the count's atomic returns it; it is stored last, so that its latency overlaps the deposit)
 __device__ __forceinline__ void deposit_runs3(const PushParams& p, int s, bool alive, const int* c, const float* t,
                                               int old, unsigned* wq, int* hist, int* rank) {
     const int lane = threadIdx.x & 31;
@@ -686,7 +686,7 @@ __device__ __forceinline__ void deposit_runs3(const PushParams& p, int s, bool a
             a = e + 1;
         }
     }
-    if (hist) {
+    if (rank) {
         number = __shfl_sync(FULL, number, first);
         if (alive) *rank = mover ? number : number + __popc(mine & ((1u << lane) - 1u));
     }
@@ -748,6 +748,7 @@ __global__ void __launch_bounds__(PD_THREADS, 3) push3d_direct_kernel(PushParams
         long long ke = 0;
         int i = lo + (int)threadIdx.x;
         int* hist = p.hist ? p.hist + (size_t)s * p.n[0] * p.n[1] * p.n[2] : nullptr;
+        int* rank = p.hist && p.rank ? p.rank + b0 : nullptr;
         int ncw = -1;
         float nt[3] = {0.f, 0.f, 0.f}, nv[3] = {0.f, 0.f, 0.f};
         // the source index is loaded two iterations ahead and the state one, so that neither load
@@ -785,7 +786,7 @@ __global__ void __launch_bounds__(PD_THREADS, 3) push3d_direct_kernel(PushParams
             store_state3(active, cellq + slot, alive ? (cn[0] | (cn[1] << 10) | (cn[2] << 20)) : -1, tq1 + slot,
                          tq1 + T + slot, tq1 + 2 * T + slot, tn, vq1 + slot, vq1 + T + slot, vq1 + 2 * T + slot, v);
             const int old = active ? (cw & 1023) + ((cw >> 10) & 1023) * p.hs1 + (cw >> 20) * p.hs2 : -1;
-            deposit_runs3(p, s, alive, cn, tn, old, wq, hist, p.rank + b0 + slot);  // a6
+            deposit_runs3(p, s, alive, cn, tn, old, wq, hist, rank ? rank + slot : nullptr);  // a6
         }
         ke = warp_sum_ll(ke);
         if ((threadIdx.x & 31) == 0 && ke) atomicAdd((unsigned long long*)&p.ctr->ke_fp[s], (unsigned long long)ke);
@@ -861,8 +862,10 @@ int launch_push3d_t(cpic_run* r, const PushParams& p) {
 
 // whether the 3D push the run takes is the direct kernel (see push_fused_ok)
 bool push3d_direct_taken(const cpic_run* r) {
-    if (r->D != 3 || r->magnetized || r->push_tile) return false;
-    const int k0 = r->cfg.particle_bc[0], k1 = r->cfg.particle_bc[2], k2 = r->cfg.particle_bc[4];
+    return r->D == 3 && !r->magnetized && !r->push_tile && push3d_special(r->cfg);
+}
+bool push3d_special(const cpic_config& c) {
+    const int k0 = c.particle_bc[0], k1 = c.particle_bc[2], k2 = c.particle_bc[4];
     return (k0 == K_ABS && k1 == K_REF && k2 == K_PER) || (k0 == K_PER && k1 == K_PER && k2 == K_PER);
 }
 

@@ -8,7 +8,8 @@
 // group reserves consecutive slots; the order inside a cell is unspecified) -> gather of the
 // particle data into the other buffer in slot order -> live counts. At the end of a step whose
 // push and injection numbered the particles of each cell, only the scan and a look-up of the
-// slot are left (place_kernel), and the gather is the next push's.
+// slot are left (place_kernel), and the gather is the next push's; a run without room for the
+// numbers (see numbers_particles) has the push's counts and the rank pass.
 #include "particles.cuh"
 
 namespace cpic {
@@ -427,6 +428,18 @@ __global__ void __launch_bounds__(256) place_kernel(SortParams p, const int* __r
     p.ctr->perm = 1;
 }
 
+// After a counted step of a run without room for the numbers, behind the rank pass: the live counts
+// become the sorted ones and the order is left pending, as by place_kernel.
+__global__ void sort_fused_finish_kernel(SortParams p) {
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    for (int sp = 0; sp < p.nsp; ++sp) {
+        const long long cnt = p.scan[(long long)(sp + 1) * p.ncell] - p.scan[(long long)sp * p.ncell];
+        p.ctr->count[sp] = cnt;
+        p.ctr->alive[sp] = cnt;
+    }
+    p.ctr->perm = 1;
+}
+
 SortParams sort_params(cpic_run* r) {
     SortParams p;
     p.D = r->D;
@@ -475,7 +488,7 @@ int launch_sort(cpic_run* r, bool fused) {
     if (pblocks > 8LL * device_sm_count()) pblocks = 8LL * device_sm_count();
     if (pblocks < 1) pblocks = 1;
     if (fused && !r->count_hist) {
-        set_error("the step has not numbered its particles");
+        set_error("the step has not counted its particles");
         return CPIC_ERR_STATE;
     }
     r->count_hist = false;
@@ -497,7 +510,7 @@ int launch_sort(cpic_run* r, bool fused) {
     }
     scan_final_kernel<<<nb, SCAN_THREADS, 0, r->stream>>>(r->hist, N, chunk, nb > 1 ? r->scan_blocks : nullptr, r->scan);
     CPIC_CHECK_LAUNCH();
-    if (fused) {
+    if (fused && r->prank) {
         long long most = 0;
         for (int s = 0; s < p.nsp; ++s) most = r->pb.capacity[s] > most ? r->pb.capacity[s] : most;
         long long nb = (most + 1023) / 1024, cap = 8LL * device_sm_count() / p.nsp;
@@ -515,6 +528,12 @@ int launch_sort(cpic_run* r, bool fused) {
     else
         rank_kernel<3><<<(int)pblocks, 256, 0, r->stream>>>(p);
     CPIC_CHECK_LAUNCH();
+    if (fused) {
+        sort_fused_finish_kernel<<<1, 32, 0, r->stream>>>(p);
+        CPIC_CHECK_LAUNCH();
+        r->order_pending = true;
+        return CPIC_OK;
+    }
     return launch_gather(r, p);
 }
 

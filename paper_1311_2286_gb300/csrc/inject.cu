@@ -95,7 +95,8 @@ __device__ float drift_normal_speed(double q, double u, double vth) {
             v -= (F(v) - q) / f;
             // one step leaves the square of the FP32 part's error
             const double w = it == 0 ? fmax(10.0 * m / f, 1e-11 * vth) : 10.0 * m / f;
-            if (v - w > lo && v + w < hi && F(v - w) < q - m && F(v + w) > q + m) {
+            // (far out of the domain z is all rounding, and where it is not positive m says nothing)
+            if (F.z > 0.0 && v - w > lo && v + w < hi && F(v - w) < q - m && F(v + w) > q + m) {
                 a = v - w;
                 b = v + w;
                 if ((float)(a - last) == (float)(b + last)) return (float)a;

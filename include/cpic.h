@@ -308,8 +308,11 @@ int cpic_inject(cpic_run* run);
 /* a7: counting sort of every species by cell (row-major cell index), dropping dead slots. */
 int cpic_sort(cpic_run* run);
 /* a9: RHS from the charge grids (Omega_c Q_c plus Dirichlet terms), then multigrid
- * V-cycles (Sec. II.B.3) until ||r||/||b|| <= rtol or max_cycles; synchronises once per
- * cycle. cycles, residual: host, may be NULL. CPIC_ERR_NOT_CONVERGED if rtol was not met. */
+ * V-cycles (Sec. II.B.3) until ||r||/||b|| <= rtol or max_cycles; synchronises, once per
+ * cycle where no single kernel holds the solve. b = 0 is within any tolerance; a residual that is
+ * not a number never is. cycles, residual: host, may be NULL. CPIC_ERR_NOT_CONVERGED if rtol was
+ * not met, CPIC_ERR_TIMEOUT if a kernel's bounded wait for its data ran out (phi is then not
+ * valid). */
 int cpic_solve_field(cpic_run* run, double rtol, int max_cycles, int* cycles, double* residual);
 
 /* Outer iteration of the field solve on the kernel-chain path (3D runs, and 2D runs that the
@@ -326,7 +329,8 @@ int cpic_solve_field(cpic_run* run, double rtol, int max_cycles, int* cycles, do
  *                         the result's accuracy are the same; mg_cycles counts V-cycles.
  *                         A grid whose levels all fit one CTA's shared memory (point
  *                         smoothing, bilinear prolongation) runs the whole solve as one
- *                         kernel, with the same operations.
+ *                         kernel, with the same operations (its FP64 sums in another
+ *                         order).
  * Invalidates the run's captured step graphs. CPIC_ERR_INVALID for another value. */
 #define CPIC_SOLVER_MG 0
 #define CPIC_SOLVER_BICGSTAB 1

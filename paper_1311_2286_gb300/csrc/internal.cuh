@@ -314,8 +314,6 @@ bool push2d_batchable(const cpic_run* r);
 int enqueue_step_pre(cpic_run* r, bool with_push);
 int enqueue_step_post(cpic_run* r, bool sort, bool finalized, bool fused_sort = false);
 int launch_push3d(cpic_run* r, const PushParams& p);  // CPIC_ERR_NOT_BUILT: no specialisation
-// one PIC step without the field solve, enqueued on r->stream (also inside stream capture)
-int enqueue_step(cpic_run* r, bool sort);
 int count_kernel_nodes(cudaGraph_t g, int* out);
 int launch_load_maxwellian(cpic_run* r, int sp, long long n, double vth, const double* drift, unsigned long long seed);
 // inject.cu

@@ -735,8 +735,8 @@ __device__ __forceinline__ int ring_of(const TilePair& t, int p) {
     return max(max(TL_H - x, x - TL_H - TL_X + 1), max(max(TL_H - r, r - TL_H - TL_Y + 1), 0));
 }
 
-// Down: x = 0, sweeps of colours 0, 1, 0, 1, then Cl.b = sums of the residuals, in the order of
-// restrict_at. x keeps the first colour only: the way up prolongs onto it and relaxes the
+// Down: x = 0, sweeps of colours 0, 1, 0, 1, then Cl.b = sums of the residuals, in
+// restrict_kernel's order. x keeps the first colour only: the way up prolongs onto it and relaxes the
 // second from it.
 __global__ void __launch_bounds__(TL_THREADS) level_down2_kernel(const __grid_constant__ LV<float> L, float* bc, int cn0) {
     __shared__ float x[(TL_R + 2) * TL_W + 2];
@@ -900,7 +900,7 @@ __device__ __forceinline__ void cta_sweep(const CtaLevel& L, int colour, bool fi
     __syncthreads();
 }
 
-// Cl.b = sum of the children's residuals, in the order of restrict_at
+// Cl.b = sum of the children's residuals, in restrict_kernel's order
 template <int D, int NPT>
 __device__ __forceinline__ void cta_restrict(const CtaLevel& F, const CtaLevel& Cl) {
     for (int C = threadIdx.x; C < Cl.ncell; C += blockDim.x) {
@@ -1218,7 +1218,7 @@ __global__ void __launch_bounds__(512, 1) coarse_cluster_kernel(const __grid_con
                 slab_sweep(L, col, it == 0 && col == 0);
                 cl.sync();
             }
-        // restriction, in the order of restrict_at: to this CTA's planes of a split level, or to every
+        // restriction, in restrict_kernel's order: to this CTA's planes of a split level, or to every
         // CTA's copy of the first level held whole
         const bool whole = t == P.ns - 1;
         const int cn0 = L.half, cn1 = L.n1 / 2, cplane = cn0 * cn1, cells = L.R / 2 * cplane, nc = L.R * L.plane;
@@ -2639,8 +2639,8 @@ int mg_setup(cpic_run* r) {
     return prepare_slabs(r, &r->slab_cs);
 }
 
-// Stream-ordered solve; the host reads the device decision after every cycle
-// (cpic_solve_field and the steps of an uncaptured cpic_step).
+// Stream-ordered solve (cpic_solve_field and the steps of an uncaptured cpic_step); where no single
+// kernel holds the loop, the host reads the device's decision after every cycle.
 int mg_solve(cpic_run* r, double rtol, int max_cycles, bool fold, int* cycles, double* res) {
     LVSet S = make_set(r);
     CtaSolve one;

@@ -105,15 +105,13 @@ __device__ __forceinline__ void pair_sub(float& h, float& l, float ah, float al,
     l = __fadd_rn(l, __fsub_rn(e, pe));
 }
 
-// What a phase knows of its CTA: the slab's neighbours and the run's flags
-struct Ctx {
-    float* sm;
-    float *lower, *upper;  // the neighbours' shared memory (null outside the domain)
-    int per0, per1;
+// the shared memory of the CTAs whose slabs lie below and above (null outside the domain)
+struct Neighbours {
+    float *lower, *upper;
 };
 
 // a value at offset off of slab row rr into the halo rows of the neighbours, h rows deep (h <= R)
-__device__ __forceinline__ void send(const Ctx& X, int off, int rr, int R, int n0, int h, float v) {
+__device__ __forceinline__ void send(const Neighbours& X, int off, int rr, int R, int n0, int h, float v) {
     if (rr < h && X.lower) X.lower[off + R * n0] = v;
     if (rr >= R - h && X.upper) X.upper[off - R * n0] = v;
 }
@@ -258,10 +256,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) mg_cluster_kernel(const __grid_
     float *rl = sm + P.orl, *eh = sm + P.oeh, *el = sm + P.oel, *rs = sm + P.ors;
     double* part = reinterpret_cast<double*>(sm + P.opart);  // [2][16][2]
     float* partf = sm + P.opart + 128;                       // [2][16]
-    Ctx X;
-    X.sm = sm;
-    X.per0 = P.per0;
-    X.per1 = P.per1;
+    Neighbours X;
     X.lower = rank > 0 ? cl.map_shared_rank(sm, rank - 1) : (P.per1 ? cl.map_shared_rank(sm, cs - 1) : nullptr);
     X.upper = rank < cs - 1 ? cl.map_shared_rank(sm, rank + 1) : (P.per1 ? cl.map_shared_rank(sm, 0) : nullptr);
 
@@ -653,7 +648,9 @@ struct ClusterPlan {
     ClParams P;
 };
 
-constexpr size_t CL_SMEM_MAX = 225 * 1024;  // of the 227 KB a CTA may have; the rest is static
+// an upper bound, of the 227 KB a CTA may have; mg_cluster_prepare asks the device what the kernel's
+// static memory leaves
+constexpr size_t CL_SMEM_MAX = 225 * 1024;
 
 // cs CTAs with nd split levels; false where the slabs do not come out even or do not fit
 bool plan_cluster(const cpic_run* r, int cs, int nd, ClusterPlan* out) {
@@ -766,6 +763,7 @@ int mg_cluster_prepare(cpic_run* r) {
         for (int nd = 1; nd < r->nlevels; ++nd) {
             ClusterPlan plan;
             if (!plan_cluster(r, cs, nd, &plan)) continue;
+            // (a larger cluster or another split level for less than the model can tell, 3 %, is not taken)
             if ((int)plan.smem > dyn_max || (r->cluster_cs && plan.cost >= 0.97 * best)) continue;
             cudaLaunchConfig_t cfg = {};
             cudaLaunchAttribute attr[1];

@@ -148,8 +148,8 @@ int cpic_query_footprint(const cpic_config* cfg, size_t* device_bytes);
 
 /* Create a run on the current device. arena: NULL (the run cudaMallocs its memory) or a
  * device buffer of at least cpic_query_footprint bytes, 256-byte aligned, owned by the
- * caller (one that is short of the sort's numbers only is taken, as is a device whose memory is:
- * the run then sorts without them). stream: cudaStream_t to enqueue on (NULL = legacy default stream). */
+ * caller (a device whose memory is short of the sort's numbers only gives a run that sorts without
+ * them). stream: cudaStream_t to enqueue on (NULL = legacy default stream). */
 int cpic_create(const cpic_config* cfg, void* arena, size_t arena_bytes, void* stream,
                 cpic_run** out);
 /* The run's configuration as in use (the sort interval as last chosen by cpic_autotune). */
@@ -447,7 +447,8 @@ int cpic_set_push_tuning(cpic_run* run, int chunk, int tile);
  * a run that changed its components after cpic_set_floating continues to the solve
  * tolerance instead. */
 int cpic_checkpoint(cpic_run* run, const char* path);
-/* Creates a run from a checkpoint (arena/stream as in cpic_create); stepping it continues
+/* Creates a run from a checkpoint (arena/stream as in cpic_create; an arena as large as the saved
+ * run's will do); stepping it continues
  * the saved run exactly (particles, charge, potential and diagnostics bit for bit).
  * CPIC_ERR_INVALID for a missing, foreign or truncated file. */
 int cpic_restore(const char* path, void* arena, size_t arena_bytes, void* stream, cpic_run** out);

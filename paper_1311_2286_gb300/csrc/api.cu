@@ -818,6 +818,87 @@ int step_once(cpic_run* r, bool solve) {
 }
 
 }  // namespace
+
+int create_run(const cpic_config* cfg, void* arena, size_t arena_bytes, void* stream, bool numbers_optional,
+               cpic_run** out) {
+    if (!out) {
+        set_error("out is NULL");
+        return CPIC_ERR_INVALID;
+    }
+    *out = nullptr;
+    int st = validate(cfg);
+    if (st) return st;
+    cpic_run* r = new cpic_run;
+    memset(r, 0, sizeof(*r));
+    r->solver = CPIC_SOLVER_BICGSTAB;
+    r->floating_face = -1;
+    r->kick_fraction = 1.0;
+    r->push_tile = 1;
+    init_geometry_sizes(r, cfg);
+    st = setup_levels(r);
+    if (st) {
+        delete r;
+        return st;
+    }
+    r->stream = (cudaStream_t)stream;
+    auto planned = [&](bool numbered) {
+        r->numbered = numbered;
+        Planner dry;
+        plan(r, dry);
+        return dry.used + 256;
+    };
+    size_t need = planned(numbers_particles(*cfg));
+    if (arena && arena_bytes < need && r->numbered && numbers_optional) need = planned(false);
+    if (arena) {
+        if (arena_bytes < need || (reinterpret_cast<uintptr_t>(arena) & 255)) {
+            set_error("arena too small or misaligned: need %zu bytes, 256-byte aligned", need);
+            delete r;
+            return CPIC_ERR_OOM;
+        }
+        r->arena = (char*)arena;
+        r->own_memory = false;
+    } else {
+        void* p = nullptr;
+        cudaError_t e = cudaMalloc(&p, need);
+        if (e == cudaErrorMemoryAllocation && r->numbered) {
+            (void)cudaGetLastError();
+            need = planned(false);
+            e = cudaMalloc(&p, need);
+        }
+        if (e != cudaSuccess) {
+            set_error("cudaMalloc(%zu) failed: %s", need, cudaGetErrorString(e));
+            delete r;
+            return CPIC_ERR_OOM;
+        }
+        r->arena = (char*)p;
+        r->own_memory = true;
+    }
+    r->arena_bytes = need;
+    Planner P;
+    P.base = r->arena;
+    plan(r, P);
+    cudaError_t e = cudaMemsetAsync(r->ctr, 0, sizeof(DevCounters), r->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(r->charge, 0, sizeof(unsigned long long) * r->ncell * cfg->n_species, r->stream);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(r->charge_h, 0, sizeof(unsigned long long) * r->ncell_h * cfg->n_species, r->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(r->pb.cell[0], 0xff, sizeof(int) * r->pb.total, r->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(r->pb.cell[1], 0xff, sizeof(int) * r->pb.total, r->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(r->ticket, 0, sizeof(unsigned) * 4, r->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(r->kry, 0, sizeof(KrylovState), r->stream);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(r->collect, 0, sizeof(unsigned long long) * cfg->n_species * 2 * r->ncollect, r->stream);
+    if (e != cudaSuccess) {
+        st = cuda_fail(e, "initial memset", __FILE__, __LINE__);
+        if (r->own_memory) cudaFree(r->arena);
+        delete r;
+        return st;
+    }
+    r->prof_events = new std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>>();
+    r->prof_pool = new std::vector<cudaEvent_t>();
+    *out = r;
+    return CPIC_OK;
+}
+
 }  // namespace cpic
 
 using namespace cpic;
@@ -935,83 +1016,7 @@ int cpic_set_push_tuning(cpic_run* r, int chunk, int tile) {
 }
 
 int cpic_create(const cpic_config* cfg, void* arena, size_t arena_bytes, void* stream, cpic_run** out) {
-    if (!out) {
-        set_error("out is NULL");
-        return CPIC_ERR_INVALID;
-    }
-    *out = nullptr;
-    int st = validate(cfg);
-    if (st) return st;
-    cpic_run* r = new cpic_run;
-    memset(r, 0, sizeof(*r));
-    r->solver = CPIC_SOLVER_BICGSTAB;
-    r->floating_face = -1;
-    r->kick_fraction = 1.0;
-    r->push_tile = 1;
-    init_geometry_sizes(r, cfg);
-    st = setup_levels(r);
-    if (st) {
-        delete r;
-        return st;
-    }
-    r->stream = (cudaStream_t)stream;
-    auto planned = [&](bool numbered) {
-        r->numbered = numbered;
-        Planner dry;
-        plan(r, dry);
-        return dry.used + 256;
-    };
-    size_t need = planned(numbers_particles(*cfg));
-    // the numbers are left out where only they do not fit
-    if (arena && arena_bytes < need && r->numbered) need = planned(false);
-    if (arena) {
-        if (arena_bytes < need || (reinterpret_cast<uintptr_t>(arena) & 255)) {
-            set_error("arena too small or misaligned: need %zu bytes, 256-byte aligned", need);
-            delete r;
-            return CPIC_ERR_OOM;
-        }
-        r->arena = (char*)arena;
-        r->own_memory = false;
-    } else {
-        void* p = nullptr;
-        cudaError_t e = cudaMalloc(&p, need);
-        if (e == cudaErrorMemoryAllocation && r->numbered) {
-            (void)cudaGetLastError();
-            need = planned(false);
-            e = cudaMalloc(&p, need);
-        }
-        if (e != cudaSuccess) {
-            set_error("cudaMalloc(%zu) failed: %s", need, cudaGetErrorString(e));
-            delete r;
-            return CPIC_ERR_OOM;
-        }
-        r->arena = (char*)p;
-        r->own_memory = true;
-    }
-    r->arena_bytes = need;
-    Planner P;
-    P.base = r->arena;
-    plan(r, P);
-    cudaError_t e = cudaMemsetAsync(r->ctr, 0, sizeof(DevCounters), r->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->charge, 0, sizeof(unsigned long long) * r->ncell * cfg->n_species, r->stream);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(r->charge_h, 0, sizeof(unsigned long long) * r->ncell_h * cfg->n_species, r->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->pb.cell[0], 0xff, sizeof(int) * r->pb.total, r->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->pb.cell[1], 0xff, sizeof(int) * r->pb.total, r->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->ticket, 0, sizeof(unsigned) * 4, r->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->kry, 0, sizeof(KrylovState), r->stream);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(r->collect, 0, sizeof(unsigned long long) * cfg->n_species * 2 * r->ncollect, r->stream);
-    if (e != cudaSuccess) {
-        st = cuda_fail(e, "initial memset", __FILE__, __LINE__);
-        if (r->own_memory) cudaFree(r->arena);
-        delete r;
-        return st;
-    }
-    r->prof_events = new std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>>();
-    r->prof_pool = new std::vector<cudaEvent_t>();
-    *out = r;
-    return CPIC_OK;
+    return create_run(cfg, arena, arena_bytes, stream, false, out);
 }
 
 int cpic_destroy(cpic_run* r) {

@@ -271,6 +271,10 @@ struct cpic_run {
 
 namespace cpic {
 // ---------------------------------------------------------------- launchers (per .cu)
+// api.cu
+// cpic_create; numbers_optional: an arena that is short of the particles' numbers only is taken,
+// without them (a restored run's arena may be from before it was given a sort interval)
+int create_run(const cpic_config* cfg, void* arena, size_t arena_bytes, void* stream, bool numbers_optional, cpic_run** out);
 // geometry.cu
 int launch_map_analytic(cpic_run* r, int map_id, const double* params, int nparams);
 int launch_geometry(cpic_run* r);

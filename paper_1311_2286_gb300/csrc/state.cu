@@ -274,7 +274,7 @@ int cpic_restore(const char* path, void* arena, size_t arena_bytes, void* stream
         return CPIC_ERR_INVALID;
     }
     cpic_run* r = nullptr;
-    int st = cpic_create(&cfg, arena, arena_bytes, stream, &r);
+    int st = create_run(&cfg, arena, arena_bytes, stream, true, &r);
     if (st) {
         fclose(f);
         return st;

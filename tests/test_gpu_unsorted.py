@@ -1,5 +1,7 @@
 """Pushes of particles that are not in cell order: the deposit's other branch in 3D, and the steps
 that do not count for a sort in 2D."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -52,28 +54,36 @@ def test_any_order_gives_the_same_particles_and_charge(cpic, grid, kind):
 
 
 @pytest.mark.parametrize("grid", [(12, 20, 8), (72, 40)])
-def test_a_run_without_room_for_the_numbers_sorts_all_the_same(cpic, grid):
-    """An arena that has no room for the particles' numbers is taken, and a run made without a sort
-    interval may be given one: the particles and their order by cell are those of a run with numbers."""
+def test_a_run_without_room_for_the_numbers_sorts_all_the_same(cpic, grid, tmp_path):
+    """A run made without a sort interval may be given one, and restored into its arena from then: the
+    particles and their order by cell are those of a run with room for the numbers. (A new run with
+    an interval needs that room.)"""
     torch = pytest.importorskip("torch")
     mk = wl.sphere if len(grid) == 3 else wl.cylinder
     got = []
-    for how in ("numbers", "small_arena", "interval_later"):
+    for how in ("numbers", "interval_later", "restored"):
         w = mk(*grid, npart_per_species=20_001, inject=True)
         small = cpic.Run.footprint(cpic.config_from_workload(w, sort_interval=0))
         arena = torch.empty(small, dtype=torch.uint8, device="cuda") if how != "numbers" else None
-        run = cpic.run_from_workload(w, sort_interval=0 if how == "interval_later" else 1, arena=arena)
-        if how == "interval_later":
+        run = cpic.run_from_workload(w, sort_interval=1 if how == "numbers" else 0, arena=arena)
+        if how != "numbers":
             run.set_sort_interval(1)
         run.set_push_tuning(0, 0)
         run.set_phi(wl.random_field(np.random.default_rng(4), tuple(reversed(run.n)), 0.5))
-        run.step_particles(3)
+        run.step_particles(2)
+        if how == "restored":
+            run.checkpoint(str(tmp_path / "state"))
+            run.close()
+            run.h = ctypes.c_void_p()
+            cpic.check(cpic.load().cpic_restore(str(tmp_path / "state").encode(), ctypes.c_void_p(arena.data_ptr()),
+                                                small, None, ctypes.byref(run.h)))
+            run.set_push_tuning(0, 0)
+        run.step_particles(1)
         got.append([(run.particles(s)[0], _records(run, s), run.charge(s)) for s in range(2)])
         run.close()
     for other in got[1:]:
         for a, b in zip(got[0], other):
             assert all(np.array_equal(x, y) for x, y in zip(a, b))
     with pytest.raises(cpic.CpicError) as e:
-        cpic.Run(cpic.config_from_workload(w, sort_interval=1), arena=torch.empty(small - 256, dtype=torch.uint8,
-                                                                                 device="cuda"))
+        cpic.Run(cpic.config_from_workload(w, sort_interval=1), arena=arena)
     assert e.value.status == -2

@@ -220,7 +220,7 @@ struct cpic_run {
     bool graph_sort_fused[2][2];       // the graph's sort leaves its order to the next push
     cudaStream_t capture_stream;
     int* done_host;              // page-locked: the done flags of the last two cycles (mg_solve), and
-    cudaEvent_t done_event[2];   // the events after them; created when first needed
+    cudaEvent_t done_event[2];   // the events after them; grids of the cluster class without a layout
     int cluster_cs;              // cluster size of the cluster solver (0: not applicable)
     int cluster_nd;              // its split levels
     bool cluster_class;          // V-cycles are the outer iteration, also where no cluster layout fits

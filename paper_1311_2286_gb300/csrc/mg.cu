@@ -2648,12 +2648,9 @@ int mg_solve(cpic_run* r, double rtol, int max_cycles, bool fold, int* cycles, d
     // some 40 us, and a host that waits for each adds half as much: they are kept one cycle ahead,
     // with the decision written straight to host memory, and what is enqueued beyond the last one
     // leaves phi and the counters alone. (Larger grids lose more by that cycle than by the waits.)
-    // 192 x 128, 15 cycles: 850 us, 1009 with a copy and a wait a cycle; 256 x 64, 90: 4229 and 5583.
+    // 192 x 128, 15 cycles: 850 to 903 us, 1009 with a copy and a wait a cycle; 256 x 64, 90: 4229 to
+    // 4454 and 5583.
     const bool ahead = max_cycles > 0 && r->cluster_class && !r->cluster_cs;
-    if (ahead && !r->done_host) {
-        CPIC_CUDA(cudaHostAlloc((void**)&r->done_host, 2 * sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped));
-        for (int k = 0; k < 2; ++k) CPIC_CUDA(cudaEventCreateWithFlags(&r->done_event[k], cudaEventDisableTiming));
-    }
     auto told = [&](int cyc) { return ahead ? r->done_host + (cyc & 1) : nullptr; };
     auto mark = [&](int cyc) -> int {
         CPIC_CUDA(cudaEventRecord(r->done_event[cyc & 1], r->stream));

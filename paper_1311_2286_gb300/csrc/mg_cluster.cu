@@ -778,7 +778,13 @@ int mg_cluster_prepare(cpic_run* r) {
             r->cluster_nd = nd;
             best = plan.cost;
         }
-    if (!r->cluster_cs) return CPIC_OK;
+    if (!r->cluster_cs) {
+        if (!r->done_host) {  // (set up with the map: a solve allocates nothing)
+            CPIC_CUDA(cudaHostAlloc((void**)&r->done_host, 2 * sizeof(int), cudaHostAllocPortable | cudaHostAllocMapped));
+            for (int k = 0; k < 2; ++k) CPIC_CUDA(cudaEventCreateWithFlags(&r->done_event[k], cudaEventDisableTiming));
+        }
+        return CPIC_OK;
+    }
     const long long nb = (r->ncell + 255) / 256;
     split_operator_kernel<<<(int)(nb < 1024 ? nb : 1024), 256, 0, r->stream>>>(
         r->lev[0].A, reinterpret_cast<float*>(r->kv), r->n[0], r->n[1], r->cfg.field_bc[0] == CPIC_BC_PERIODIC,
